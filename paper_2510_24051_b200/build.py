@@ -36,7 +36,7 @@ def sources():
 
 def _digest():
     h = hashlib.sha256(" ".join(NVCC_FLAGS).replace(ROOT, "").encode())
-    files = sources() + sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".h"))
+    files = sources() + sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh")))
     files += [os.path.join(INCLUDE, f) for f in sorted(os.listdir(INCLUDE))]
     for f in files:
         h.update(os.path.basename(f).encode())

@@ -7,7 +7,7 @@
 //   * attn_tile_kernel  - row tiles (prefill chunks, token trees): each consumer warp owns 16
 //     query rows and every warp walks the same page stream filled by a producer warp.
 //   * merge_kernel                 - LSE-weighted merge of split partials.
-//   * simple_kernel                - plain CUDA-core kernel (fp32 pools and shapes the tile
+//   * simple_kernel                - plain CUDA-core kernel (PIE_PLAN_FORCE_SIMPLE, shapes the tile
 //     kernels do not cover); one warp per (token, head) row, sequential online softmax.
 #include <cuda_bf16.h>
 
@@ -1179,6 +1179,7 @@ int pie_launch_split(pie_ctx* ctx, const pie_plan* plan, const void* q, const vo
   p.k_new = k_new;
   p.v_new = v_new;
   const int D = ctx->cfg.head_dim, P = ctx->cfg.page_size, n = plan->split.grid, ni = (int)plan->split.items.size();
+  if (ctx->cfg.dtype == PIE_DTYPE_F32) return pie_launch_f32(ctx, p, n, plan->split.slot_rows, false, s);
   // ring depth: 128 - 192 KB of copies in flight per SM (measured on the 64-request decode batch with 4 KB stages:
   // depths 3 and 4 run 1.5 % faster than 5 and 6 - a deeper ring only lengthens the queue in front of every copy)
   if (plan->split.heads_per_unit == 2) {   // units of two adjacent kv heads: copies of 8 KB instead of 4 KB (of 4 KB instead of 2 KB)
@@ -1198,6 +1199,7 @@ int pie_launch_split(pie_ctx* ctx, const pie_plan* plan, const void* q, const vo
 int pie_launch_tiles(pie_ctx* ctx, const pie_plan* plan, const void* q, void* out, float* lse, cudaStream_t s) {
   AttnParams p = make_params(ctx, plan, plan->tile, q, out, lse);
   const int D = ctx->cfg.head_dim, P = ctx->cfg.page_size, grid = plan->tile.grid;
+  if (ctx->cfg.dtype == PIE_DTYPE_F32) return pie_launch_f32(ctx, p, grid, 64, true, s);
   if (plan->tile_tc) return pie_launch_tc_tiles(ctx, p, grid, plan->info.num_query_tokens, s);
   if (D == 64 && P == 16) return launch_tiles<64, 16, 4>(ctx, p, grid, s);
   if (D == 128 && P == 16) return launch_tiles<128, 16, 4>(ctx, p, grid, s);
@@ -1208,7 +1210,9 @@ int pie_launch_tiles(pie_ctx* ctx, const pie_plan* plan, const void* q, void* ou
 
 int pie_launch_merge(pie_ctx* ctx, const pie_plan* plan, const PieLaunchList& ll, void* out, float* lse, cudaStream_t s) {
   const int D = ctx->cfg.head_dim;
-  const bool tiles = ll.slot_rows >= 32;      // groups of row-tile partials: one block per group
+  // groups of row-tile partials: one block per group - when there are groups for every SM; a few groups (one long unit
+  // cut into many pieces) spread over the chip row by row instead (96 groups of 64 rows, 4 - 5 sources: 26 against 7 us)
+  const bool tiles = ll.slot_rows >= 32 && (int)ll.merges.size() >= ctx->n_sms;
   const int wpb = ll.slot_rows >= 8 ? 8 : 4;  // warps (= rows) per block
   const dim3 n((unsigned)ll.merges.size(), tiles ? 1u : (unsigned)((ll.slot_rows + wpb - 1) / wpb));
 #define PIE_MERGE(T, DD)                                                                                                   \

@@ -209,6 +209,7 @@ struct pie_ctx {
   struct HeldPages { cudaEvent_t done; std::vector<int32_t> pages; };
   std::vector<HeldPages> held_pages;
   std::vector<cudaEvent_t> held_events;   // recycled events of held_pages
+  bool f32_configured[3] = {false, false, false};   // (items of <= 4, <= 16, 64 rows)
   bool tc_configured = false, split_configured = false, split_pair_configured = false, tile_configured = false, nd_configured = false;   // kernel attributes set for this context's device
   // The block-local work list of the latest decode batch.  Consecutive steps of a serving loop bring the same
   // requests with the same page counts (a request grows by a page every page_size steps), and then the list is
@@ -284,6 +285,9 @@ bool pie_split_supported(const pie_ctx* ctx);
 bool pie_split_pair_supported(const pie_ctx* ctx);   // ... with units of two adjacent kv heads
 int pie_split_warps_per_block(const pie_ctx* ctx);
 bool pie_tc_supported(const pie_ctx* ctx);
+// fp32 pools (attn_f32_kernel.cu): one launch list; tiles: items of 64 rows, else of at most max_rows <= 16
+int pie_launch_f32(pie_ctx* ctx, const AttnParams& p, int grid, int max_rows, bool tiles, cudaStream_t s);
+int pie_f32_blocks_per_sm(const pie_ctx* ctx, bool tiles);
 // n_tokens: rows of the Q tensor (the batch's query tokens), for the bounds of the Q tensor map
 int pie_launch_tc_tiles(pie_ctx* ctx, const AttnParams& p, int grid, int64_t n_tokens, cudaStream_t s);
 

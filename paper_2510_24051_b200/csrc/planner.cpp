@@ -222,7 +222,7 @@ PieItem make_item(const Unit& u, int32_t page_begin, int32_t page_end) {
 //  * Otherwise: contiguous equal shares; a unit cut by a share boundary becomes several items
 //    whose fp32 partials are merged.
 void partition(const std::vector<Unit>& units, int grid_max, int min_pages_per_cta, int slot_rows,
-               bool allow_whole_units, PieLaunchList& ll, UnitSlots* slots_out = nullptr) {
+               bool allow_whole_units, PieLaunchList& ll, UnitSlots* slots_out = nullptr, int slack_pages = 200) {
   if (slots_out) slots_out->assign(units.size(), std::make_pair(-1, 0));
   ll.items.clear();
   ll.merges.clear();
@@ -241,8 +241,8 @@ void partition(const std::vector<Unit>& units, int grid_max, int min_pages_per_c
   ll.grid = grid;
 
   // Whole units also when there are only a few per CTA (or fewer units than CTAs), as long as dealing them out
-  // (largest first then) leaves the fullest CTA within 12 % of the average or within 200 page visits (~45 us of
-  // a row-tile CTA) of it: a cut unit costs fp32 partials of up to 256 rows, more and shorter items and the merge
+  // (largest first then) leaves the fullest CTA within 12 % of the average or within `slack_pages` page visits (200:
+  // ~45 us of a row-tile CTA) of it: a cut unit costs fp32 partials of up to 256 rows, more and shorter items and the merge
   // launch, which on a short launch is more than that imbalance (8 prefill chunks of 512 tokens: 137 -> 78 us;
   // one prompt of 2,048 tokens: 90 -> 46 us although only 64 of 148 CTAs get a unit).
   const bool many_small = (int64_t)units.size() >= 4 * (int64_t)grid && max_unit * 8 <= W / grid;
@@ -272,7 +272,7 @@ void partition(const std::vector<Unit>& units, int grid_max, int min_pages_per_c
       max_load = std::max(max_load, top.first);
       std::push_heap(heap.begin(), heap.end(), cmp);
     }
-    if (few_whole && max_load * grid * 100 > W * 112 && max_load > W / grid + 200) goto contiguous;   // too uneven: cut the units instead
+    if (few_whole && max_load * grid * 100 > W * 112 && max_load > W / grid + slack_pages) goto contiguous;   // too uneven: cut the units instead
     for (int c = 0; c < grid; ++c) ll.cta_ptr[c + 1] += ll.cta_ptr[c];
     std::vector<int32_t> fill(ll.cta_ptr.begin(), ll.cta_ptr.end() - 1);
     ll.items.resize(units.size());
@@ -1092,7 +1092,8 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
   // ---- route requests to kernels and partition the work
   // (head groups above 16 - multi-query models - do not fit the split-KV kernel's 16 rows per warp: every request
   //  of such a context has more than 16 rows and runs on the row-tile kernel)
-  const bool tiles_ok = (pie_split_supported(ctx) || (pie_tc_supported(ctx) && G > 16)) && !(b->flags & PIE_PLAN_FORCE_SIMPLE);
+  const bool f32 = cfg.dtype == PIE_DTYPE_F32;   // fp32 pools: both launch lists run on the fp32 kernel (items of at most 16 / of 64 rows)
+  const bool tiles_ok = (f32 || pie_split_supported(ctx) || (pie_tc_supported(ctx) && G > 16)) && !(b->flags & PIE_PLAN_FORCE_SIMPLE);
   std::vector<Unit> split_units, tile_units;
   plan->simple_rows.clear();
   // (8-token pages: the mma.sync row-tile kernel behind PIE_PLAN_NO_TENSOR_TILES has no instantiation, the flag is ignored)
@@ -1114,7 +1115,7 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
   struct Cascade { int32_t first, n, L, vreq; bool big; };
   std::vector<Cascade> cascades;
   std::vector<int32_t> casc_of(R, -1);
-  if (tiles_ok && !(b->flags & PIE_PLAN_NO_CASCADE) && all_rows_out) {   // (the gathered rows of a group must be consecutive query tokens)
+  if (tiles_ok && !f32 && !(b->flags & PIE_PLAN_NO_CASCADE) && all_rows_out) {   // (the gathered rows of a group must be consecutive query tokens)
     const bool always = (b->flags & PIE_PLAN_CASCADE_ALWAYS) != 0;
     const int min_n = always ? 2 : 4, min_L = always ? 1 : 16;
     auto clean_prefix = [&](const PieReq& q) {  // leading kept pages that are fully visible and in place
@@ -1283,10 +1284,21 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
       }
     }
   }
+  if (f32 && !split_units.empty() && !tile_units.empty() && ctx->options[PIE_OPT_OVERLAP] != 2) {
+    // fp32 pools: a block of each kernel fits an SM next to one of the other, and one is bound by the FMA pipe, the
+    // other by memory latency.  Fork and join cost about as much as 5 us of either (est.: 15 ns per 16-token page of a
+    // 64-row item, 3 TB/s).
+    double t_tile = 0, t_split = 0;
+    for (const Unit& u : tile_units) t_tile += (double)(u.page_end - u.page_begin) * P * cfg.head_dim * (15e-9 / 1024);
+    for (const Unit& u : split_units) t_split += (double)(u.page_end - u.page_begin) * P * cfg.head_dim * 8 / 3e12;
+    plan->overlap = ctx->options[PIE_OPT_OVERLAP] == 1 || std::min(t_tile, t_split) > 8e-6;
+  }
   // row tiles first: the cascade pieces get their partial slots, which the split units of the
   // cascaded requests then name as further sources of their merge groups
   UnitSlots tile_slots;
-  partition(tile_units, tile_sms, plan->tile_tc ? 32 : 8, TILE_ROWS, true, plan->tile, &tile_slots);
+  // (fp32: a page of 16 tokens takes a block of 64 rows about 1 us, the merge launch 4 - 5 us)
+  if (f32) partition(tile_units, tile_sms * pie_f32_blocks_per_sm(ctx, true), 4, TILE_ROWS, true, plan->tile, &tile_slots, 5);
+  else partition(tile_units, tile_sms, plan->tile_tc ? 32 : 8, TILE_ROWS, true, plan->tile, &tile_slots);
   // merge groups of the larger cascaded requests (row-tile items over their private pages): add the slots of
   // the cascade pieces that hold the same rows
   for (PieMerge& m : plan->tile.merges) {
@@ -1340,7 +1352,12 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
     const bool long_launch = kv_bytes * ctx->n_sms >= 1.6e9 * split_sms;   // (fewer SMs: the same bytes take longer)
     bool plain_units = true;
     for (const Unit& u : split_units) plain_units = plain_units && !u.force_partial;
-    if (long_launch || (W >= (int64_t)200 * n_warps && !plain_units)) {
+    if (f32) {
+      // one share per block; whole units while the fullest block stays within the merge launch of the average
+      // (a block takes a 16-token page in about 0.1 us, the launch 4 - 5 us)
+      partition(split_units, split_sms * pie_f32_blocks_per_sm(ctx, false), 16, max_rows, true, plan->split, nullptr, 45);
+      plan->split.n_static = (int32_t)plan->split.items.size();
+    } else if (long_launch || (W >= (int64_t)200 * n_warps && !plain_units)) {
       chunk_units(split_units, n_warps, plan->split);
     } else {
       // fixed equal shares, nothing left to the counter (a dynamic tail of small chunks was measured:
@@ -1464,7 +1481,7 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
   // and into its staged copy), and the append launch is dropped.
   const int no_fusion = ctx->options[PIE_OPT_NO_FUSION];
   plan->append_fused = false;
-  if (!(no_fusion & 1) && all_rows_out && ctx->cfg.rope_theta <= 0.f && !cross_read && !plan->split.items.empty() &&
+  if (!(no_fusion & 1) && !f32 && all_rows_out && ctx->cfg.rope_theta <= 0.f && !cross_read && !plan->split.items.empty() &&
       plan->tile.items.empty() && plan->simple_rows.empty()) {
     bool ok = true;
     for (int r = 0; r < R && ok; ++r) {
@@ -1508,7 +1525,7 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
   info.mask_words = (int64_t)plan->mask_words.size();
   info.workspace_bytes = ((int64_t)plan->split.n_slots * plan->split.slot_rows +
                           (int64_t)plan->tile.n_slots * plan->tile.slot_rows) * (cfg.head_dim + 1) * 4;
-  info.side_by_side_sms = plan->overlap ? plan->tile.grid : 0;
+  info.side_by_side_sms = plan->overlap ? std::min(plan->tile.grid, ctx->n_sms) : 0;
   info.split_unit_kv_heads = plan->split.items.empty() ? 1 : plan->split.heads_per_unit;
   info.reserved0 = 0;
   info.launches = (plan->pre_copies.empty() ? 0 : 1) + (plan->append_fused ? 0 : 1) + (info.num_simple_rows ? 1 : 0) + (info.num_split_items ? 1 : 0) +
