@@ -209,14 +209,15 @@ typedef struct pie_plan_info {
  * slot, or a request reads a slot that a LATER request of the batch appends: the
  * vertical-batching rule of Section 5.2; reading rows an EARLIER request appends is legal,
  * because the whole batch is appended before any request attends),
- * PIE_ERR_BATCH_TOO_LARGE, PIE_ERR_MASK.  *out is set only on success.  The upload uses
- * `stream`; the call returns after it completed. */
+ * PIE_ERR_BATCH_TOO_LARGE, PIE_ERR_MASK.  *out is set only on success.  The upload is enqueued on
+ * `stream` from memory of the library's own; forwards on any stream are ordered behind it. */
 int pie_plan_forward(pie_ctx* ctx, const pie_batch_desc* batch, void* stream, pie_plan** out);
 /* Ends the plan's life.  The context keeps a few destroyed plans - host arrays, pinned upload
  * image and device arrays - and pie_plan_forward reuses them, so a loop that plans every step
  * stops allocating after its first steps (no cudaMalloc, no cudaFree and its device-wide
  * synchronisation per batch).  The call does not wait: it marks the point behind the plan's
- * latest pie_forward on that forward's stream, and the reuse waits for that point.  Destroy a
+ * latest pie_forward on that forward's stream, and the upload of the plan that takes its memory over goes
+ * behind that point (on the GPU; the host does not wait for it).  Destroy a
  * plan only when no captured graph that holds its forward will be launched again, and before
  * the stream of its latest forward is destroyed.  pie_destroy releases the kept plans. */
 int pie_plan_destroy(pie_plan* plan);

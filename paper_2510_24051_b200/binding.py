@@ -265,6 +265,7 @@ def pie_get_next_dist(ctx, logits, top_k, out_ids, out_probs, stream=None):
     fp32 tensors [n_rows, top_k]."""
     import torch
     dtype = {torch.bfloat16: PIE_DTYPE_BF16, torch.float32: PIE_DTYPE_F32}[logits.dtype]
+    assert logits.dim() == 2
     (rows, vocab), (row_stride, one) = logits.shape, logits.stride()
     assert one == 1
     _check(lib.pie_get_next_dist(ctx, _ptr(logits), dtype, rows, vocab, row_stride, top_k,

@@ -448,6 +448,7 @@ int pie_destroy(pie_ctx* ctx) {
       if (plan->d_blob) cudaFree(plan->d_blob);
       if (plan->h_image) cudaFreeHost(plan->h_image);
       if (plan->idle) cudaEventDestroy(plan->idle);
+      if (plan->uploaded) cudaEventDestroy(plan->uploaded);
     }
     delete plan;
   }
@@ -603,8 +604,50 @@ int pie_copy_kvpage(pie_ctx* ctx, int32_t n, const int32_t* src, const int32_t* 
 // Plans are recycled: pie_plan_destroy parks up to kParkedPlans objects in the context, with their
 // host vectors, pinned image and device arrays, and pie_plan_forward takes one back.  A serving
 // loop that plans every step therefore stops allocating after its first steps: no cudaMalloc and
-// no cudaFree (with its device-wide synchronisation) per batch.
+// no cudaFree (with its device-wide synchronisation) per batch.  The oldest parked plan is taken: with up to
+// four in rotation the host plans step n + 1 while the GPU still runs step n, instead of waiting for the pinned image
+// of the one plan (small decode batches, plan + forward: 41 us a step when every plan waited for its upload).
 static const size_t kParkedPlans = 4;
+
+// The plan's pinned image may be written again once its upload is over.
+static bool upload_over(const pie_plan* plan) {
+  if (!plan->upload_pending) return true;
+  const cudaError_t e = cudaEventQuery(plan->uploaded);
+  if (e == cudaSuccess) plan->upload_pending = false;
+  else cudaGetLastError();   // (not ready)
+  return e == cudaSuccess;
+}
+static cudaError_t wait_uploaded(const pie_plan* plan) {
+  if (!plan->upload_pending) return cudaSuccess;
+  const cudaError_t e = cudaEventSynchronize(plan->uploaded);
+  if (e == cudaSuccess) plan->upload_pending = false;
+  return e;
+}
+
+// Orders a forward on `s` behind the plan's upload.
+static int order_behind_upload(pie_ctx* ctx, const pie_plan* plan, cudaStream_t s) {
+  if (!plan->upload_pending) return PIE_OK;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    cap = cudaStreamCaptureStatusNone;
+  }
+  if (cap != cudaStreamCaptureStatusNone) {
+    // the graph may be replayed on any stream, at any time: the upload has to be over, and the capture must not
+    // see the wait
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    PIE_CUDA(ctx, cudaThreadExchangeStreamCaptureMode(&mode));
+    const cudaError_t e = wait_uploaded(plan);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    PIE_CUDA(ctx, e);
+    return PIE_OK;
+  }
+  if (plan->used && upload_over(plan)) return PIE_OK;
+  unsigned long long id = 0;
+  PIE_CUDA(ctx, cudaStreamGetId(s, &id));
+  if (id != plan->upload_stream_id) PIE_CUDA(ctx, cudaStreamWaitEvent(s, plan->uploaded, 0));
+  return PIE_OK;
+}
 
 static void release_plan(pie_plan* plan) {
   if (plan->ctx) {
@@ -614,11 +657,13 @@ static void release_plan(pie_plan* plan) {
     }
     pie_plan_release_scratch(plan);
   }
-  if (plan->d_blob || plan->h_image || plan->idle) {
+  if (plan->d_blob || plan->h_image || plan->idle || plan->uploaded) {
     cudaSetDevice(plan->ctx->cfg.device);
+    wait_uploaded(plan);
     if (plan->d_blob) cudaFree(plan->d_blob);   // (synchronises: nothing can still be reading the arrays afterwards)
     if (plan->h_image) cudaFreeHost(plan->h_image);
     if (plan->idle) cudaEventDestroy(plan->idle);
+    if (plan->uploaded) cudaEventDestroy(plan->uploaded);
   }
   delete plan;
 }
@@ -627,11 +672,12 @@ int pie_plan_forward(pie_ctx* ctx, const pie_batch_desc* batch, void* stream, pi
   if (!ctx || !batch || !out) return PIE_ERR_INVALID;
   pie_plan* plan = nullptr;
   if (!ctx->parked_plans.empty()) {
-    plan = ctx->parked_plans.back();
-    ctx->parked_plans.pop_back();
-  } else {
-    plan = new (std::nothrow) pie_plan();
+    // the oldest, unless its image is still being uploaded and the rotation is not full yet
+    plan = ctx->parked_plans.front();
+    if (!upload_over(plan) && ctx->parked_plans.size() < kParkedPlans) plan = nullptr;
+    else ctx->parked_plans.erase(ctx->parked_plans.begin());
   }
+  if (!plan) plan = new (std::nothrow) pie_plan();
   if (!plan) return PIE_ERR_INVALID;
   plan->ctx = ctx;
   auto give_back = [&]() {   // the object goes back as it came: its device arrays were not touched
@@ -647,8 +693,9 @@ int pie_plan_forward(pie_ctx* ctx, const pie_batch_desc* batch, void* stream, pi
     cudaStream_t s = (cudaStream_t)stream;
     const PlanLayout L = pie_plan_layout(ctx, plan);
     cudaError_t e = cudaSetDevice(ctx->cfg.device);
-    if (e == cudaSuccess && plan->idle_pending) {   // the forward that last read the device arrays must be over
-      e = cudaEventSynchronize(plan->idle);
+    if (e == cudaSuccess) e = wait_uploaded(plan);
+    if (e == cudaSuccess && plan->idle_pending) {   // the upload goes behind the forward that last read the device arrays
+      e = cudaStreamWaitEvent(s, plan->idle, 0);
       plan->idle_pending = false;
     }
     if (e == cudaSuccess && plan->h_image_bytes < L.upload) {
@@ -669,9 +716,12 @@ int pie_plan_forward(pie_ctx* ctx, const pie_batch_desc* batch, void* stream, pi
     }
     if (e == cudaSuccess) {
       pie_plan_fill(plan, L, (uint8_t*)plan->h_image);
-      if (L.upload) e = cudaMemcpyAsync(plan->d_blob, plan->h_image, L.upload, cudaMemcpyHostToDevice, s);
+      if (!plan->uploaded) e = cudaEventCreateWithFlags(&plan->uploaded, cudaEventDisableTiming);
+      if (e == cudaSuccess && L.upload) e = cudaMemcpyAsync(plan->d_blob, plan->h_image, L.upload, cudaMemcpyHostToDevice, s);
+      if (e == cudaSuccess) e = cudaEventRecord(plan->uploaded, s);
+      if (e == cudaSuccess) e = cudaStreamGetId(s, &plan->upload_stream_id);
+      plan->upload_pending = e == cudaSuccess;
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
       ctx->cuda_error = std::string("plan upload: ") + cudaGetErrorString(e);
       release_plan(plan);
@@ -765,6 +815,8 @@ int pie_forward(pie_ctx* ctx, const pie_plan* plan, const void* q, const void* k
   if (!q || !k_new || !v_new || !out || !lse) return PIE_ERR_INVALID;
   cudaStream_t s = (cudaStream_t)stream;
   PIE_CUDA(ctx, cudaSetDevice(ctx->cfg.device));
+  int rc = plan == ctx->host_plan ? PIE_OK : order_behind_upload(ctx, plan, s);
+  if (rc) return rc;
   // (a recycled plan's device arrays are rewritten only behind the forwards that read them)
   if (plan->used && plan->last_stream != s) plan->many_streams = true;
   plan->last_stream = s;
@@ -775,8 +827,8 @@ int pie_forward(pie_ctx* ctx, const pie_plan* plan, const void* q, const void* k
     if (rc0) return rc0;
   }
   const void* q_in = q;
-  int rc = plan->append_fused ? PIE_OK  // (q stays q_in: the split-KV kernel writes the new rows itself)
-                              : timed_launch(ctx, PIE_KERNEL_APPEND, s, [&] { return pie_append_and_q(ctx, plan, q_in, k_new, v_new, s, &q); });
+  rc = plan->append_fused ? PIE_OK  // (q stays q_in: the split-KV kernel writes the new rows itself)
+                          : timed_launch(ctx, PIE_KERNEL_APPEND, s, [&] { return pie_append_and_q(ctx, plan, q_in, k_new, v_new, s, &q); });
   if (rc) return rc;
   if (!plan->simple_rows.empty() &&
       (rc = timed_launch(ctx, PIE_KERNEL_SIMPLE, s, [&] { return pie_launch_simple(ctx, plan, q, out, lse, s); })))

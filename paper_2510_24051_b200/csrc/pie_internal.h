@@ -155,6 +155,12 @@ struct pie_plan {
   size_t d_blob_bytes = 0;
   void* h_image = nullptr;          // pinned host copy of the uploaded part (pie_plan_forward)
   size_t h_image_bytes = 0;
+  // The upload is only enqueued by pie_plan_forward: `uploaded` marks its end on its stream.  A forward on that
+  // stream is ordered behind it, one on another stream waits for the event (pie_forward), and the pinned image is not
+  // written again before it.
+  cudaEvent_t uploaded = nullptr;
+  unsigned long long upload_stream_id = 0;      // (an id, not the handle: a later stream may get a destroyed one's handle)
+  mutable bool upload_pending = false;          // the event has not been seen complete yet
   // recycling (pie_plan_destroy parks the object, pie_plan_forward takes it back): the device
   // arrays may be overwritten only after the last forward that read them has finished
   mutable cudaStream_t last_stream = nullptr;   // stream of the latest pie_forward with this plan
@@ -203,7 +209,7 @@ struct pie_ctx {
   void* h_stage = nullptr;  // pinned host staging of the plan image (pie_forward_host)
   size_t h_stage_bytes = 0;
   pie_plan* host_plan = nullptr;  // reused plan object of pie_forward_host
-  std::vector<pie_plan*> parked_plans;  // destroyed plans kept for reuse: host arrays, pinned image, device arrays
+  std::vector<pie_plan*> parked_plans;  // destroyed plans kept for reuse, oldest first: host arrays, pinned image, device arrays
   // Pages a plan borrowed for requests without output KvPages go back to the free list only when the
   // forward that used them is over: they wait here behind an event recorded on that forward's stream.
   struct HeldPages { cudaEvent_t done; std::vector<int32_t> pages; };
