@@ -55,59 +55,133 @@ __global__ void append_kernel(uint8_t* __restrict__ pool, const uint8_t* __restr
   }
 }
 
-// K2: copy_kvpage (Table 1).  ops[k] = {src, dst, src_off, dst_off, ntok}; kCopySplit blocks per
-// op, 16 bytes per thread and step, four loads in flight before the first store (the copy is pure
-// latency: a page is a few tens of KB).
+// Page ids and copy operations travel as kernel parameters (up to 32 KB): a call is one launch, with no staging buffer that
+// calls on several streams would share, and no host-to-device copy in front of it (a pageable copy of a few KB cost the
+// call about 6 us of host time and 2 us on the GPU).
+template <int N>
+struct Words {
+  int32_t v[N];
+};
+
+// Rows [so, so + n) of page src to rows [dof, ..) of page dst, K and V, all heads: block y of kCopySplit takes every
+// kCopySplit-th group of 16-byte chunks, four loads in flight per thread before the first store (the copy is pure latency:
+// a page is a few tens of KB).
 constexpr int kCopySplit = 4;
-__global__ void copy_kernel(uint8_t* __restrict__ pool, const int32_t* __restrict__ ops, PoolGeom g) {
-  pie_pdl_launch_dependents();
-  pie_pdl_wait();
-  const int32_t* op = ops + blockIdx.x * 5;
-  const int src = op[0], dst = op[1], so = op[2], dof = op[3], n = op[4];
-  const int chunks = g.row_bytes >> 4;
-  const int per_tok = 2 * g.n_kv_heads * chunks;
-  const int total = n * per_tok, stride = blockDim.x * kCopySplit;
-  auto addr = [&](int i, int page, int off) -> int64_t {
-    const int t = i / per_tok, rem = i - t * per_tok;
-    const int blk = rem / chunks, c = rem - blk * chunks;  // blk = head*2 + kv
-    return (int64_t)page * g.page_bytes + (int64_t)blk * g.block_bytes + pie_chunk_offset(g.slab_bytes, off + t, c);
+__device__ __forceinline__ void copy_rows(uint8_t* __restrict__ pool, int src, int dst, int so, int dof, int n, const PoolGeom& g, int chunk_shift) {
+  const int per_blk = n << chunk_shift;                 // chunks of one block's rows
+  const int total = per_blk * 2 * g.n_kv_heads, stride = blockDim.x * kCopySplit;
+  const uint8_t* from = pool + (int64_t)src * g.page_bytes;
+  uint8_t* to = pool + (int64_t)dst * g.page_bytes;
+  const float inv = 1.f / (float)per_blk;
+  auto place = [&](int i, int& blk_off, int& t, int& c) {   // chunk i: block i / per_blk, row, chunk of the row
+    int blk = (int)((float)i * inv);                        // (exact up to one: both below 2^24)
+    int rem = i - blk * per_blk;
+    if (rem < 0) --blk, rem += per_blk;
+    if (rem >= per_blk) ++blk, rem -= per_blk;
+    blk_off = blk * g.block_bytes;
+    t = rem >> chunk_shift;
+    c = rem & ((1 << chunk_shift) - 1);
   };
   for (int i0 = blockIdx.y * blockDim.x + threadIdx.x; i0 < total; i0 += 4 * stride) {
     uint4 v[4];
+    int off[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      if (i0 + k * stride < total) v[k] = *reinterpret_cast<const uint4*>(pool + addr(i0 + k * stride, src, so));
+      if (i0 + k * stride < total) {
+        int b, t, c;
+        place(i0 + k * stride, b, t, c);
+        v[k] = *reinterpret_cast<const uint4*>(from + b + pie_chunk_offset(g.slab_bytes, so + t, c));
+        off[k] = b + pie_chunk_offset(g.slab_bytes, dof + t, c);
+      }
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      if (i0 + k * stride < total) *reinterpret_cast<uint4*>(pool + addr(i0 + k * stride, dst, dof)) = v[k];
+      if (i0 + k * stride < total) *reinterpret_cast<uint4*>(to + off[k]) = v[k];
   }
 }
 
-// Canonical [n][slot][head][D] <-> pool layout, 16 bytes per thread.
-__global__ void page_io_kernel(uint8_t* __restrict__ pool, const int32_t* __restrict__ ids, uint8_t* K,
-                               uint8_t* V, int n, int write, PoolGeom g) {
-  const int chunks = g.row_bytes >> 4;
-  const int64_t per_page = (int64_t)g.page_size * g.n_kv_heads * chunks;
-  const int64_t total = (int64_t)n * per_page * 2;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    int kv = (int)(i / ((int64_t)n * per_page));
-    int64_t j = i - (int64_t)kv * n * per_page;  // chunk index inside canonical K or V
-    int pg = (int)(j / per_page);
-    int rem = (int)(j - (int64_t)pg * per_page);
-    int slot = rem / (g.n_kv_heads * chunks);
-    rem -= slot * g.n_kv_heads * chunks;
-    int head = rem / chunks, c = rem - head * chunks;
-    uint8_t* canon = (kv ? V : K) + j * 16;
-    uint8_t* p = pool + (int64_t)ids[pg] * g.page_bytes + (int64_t)(head * 2 + kv) * g.block_bytes +
-                 pie_chunk_offset(g.slab_bytes, slot, c);
-    if (write) *reinterpret_cast<uint4*>(p) = *reinterpret_cast<const uint4*>(canon);
-    else *reinterpret_cast<uint4*>(canon) = *reinterpret_cast<const uint4*>(p);
+// K2: copy_kvpage (Table 1).  Three words per operation: src, dst, src_off | dst_off << 8 | ntok << 16.
+template <int N>
+__global__ void __launch_bounds__(256) copy_kernel(uint8_t* __restrict__ pool, const __grid_constant__ Words<N> ops, PoolGeom g, int chunk_shift) {
+  pie_pdl_launch_dependents();
+  pie_pdl_wait();
+  const int src = ops.v[blockIdx.x * 3], dst = ops.v[blockIdx.x * 3 + 1], r = ops.v[blockIdx.x * 3 + 2];
+  copy_rows(pool, src, dst, r & 255, (r >> 8) & 255, r >> 16, g, chunk_shift);
+}
+
+// The same from operations in device memory (five words each): part of a plan (requests without output KvPages).
+__global__ void __launch_bounds__(256) plan_copy_kernel(uint8_t* __restrict__ pool, const int32_t* __restrict__ ops, PoolGeom g, int chunk_shift) {
+  pie_pdl_launch_dependents();
+  pie_pdl_wait();
+  const int32_t* op = ops + blockIdx.x * 5;
+  copy_rows(pool, op[0], op[1], op[2], op[3], op[4], g, chunk_shift);
+}
+
+// Canonical [n][slot][head][D] <-> pool layout.  One block per page and K / V: the page is one contiguous run of
+// canonical chunks; a thread takes every 256th, four of them in flight.  (HBM bound; the only arithmetic left per chunk is
+// a multiplication for its slot and head, where a flat index over all pages took four 64-bit divisions.)
+template <int N>
+__global__ void __launch_bounds__(256) page_io_kernel(uint8_t* __restrict__ pool, const __grid_constant__ Words<N> ids, uint8_t* __restrict__ K,
+                                                      uint8_t* __restrict__ V, int write, PoolGeom g, int chunk_shift) {
+  pie_pdl_launch_dependents();
+  pie_pdl_wait();
+  const int kv = blockIdx.y;
+  const int per_slot = g.n_kv_heads << chunk_shift, total = g.page_size * per_slot;   // chunks
+  uint8_t* canon = (kv ? V : K) + (int64_t)blockIdx.x * total * 16;
+  uint8_t* page = pool + (int64_t)ids.v[blockIdx.x] * g.page_bytes + (int64_t)kv * g.block_bytes;
+  const float inv = 1.f / (float)per_slot;
+  auto offset = [&](int i) {
+    int slot = (int)((float)i * inv);
+    int rem = i - slot * per_slot;
+    if (rem < 0) --slot, rem += per_slot;
+    if (rem >= per_slot) ++slot, rem -= per_slot;
+    return (rem >> chunk_shift) * 2 * g.block_bytes + pie_chunk_offset(g.slab_bytes, slot, rem & ((1 << chunk_shift) - 1));
+  };
+  for (int i0 = threadIdx.x; i0 < total; i0 += 4 * 256) {
+    uint4 v[4];
+    int off[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int i = i0 + k * 256;
+      if (i < total) {
+        off[k] = offset(i);
+        v[k] = write ? reinterpret_cast<const uint4*>(canon)[i] : *reinterpret_cast<const uint4*>(page + off[k]);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int i = i0 + k * 256;
+      if (i < total) {
+        if (write) *reinterpret_cast<uint4*>(page + off[k]) = v[k];
+        else reinterpret_cast<uint4*>(canon)[i] = v[k];
+      }
+    }
   }
 }
 
-int grid_for(int64_t work_items, int threads, int n_sms) {
-  int64_t blocks = (work_items + threads - 1) / threads;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)n_sms * 8));
+int log2_exact(int x) {
+  int l = 0;
+  while ((1 << l) < x) ++l;
+  return l;
+}
+
+// Calls f(Words<N>) with `n` words (`word(i)` each) copied into the smallest parameter block that holds them.
+constexpr int kMaxWords = 8000;   // (32,764 bytes of parameters per launch, less the other arguments)
+template <class Word, class F>
+int with_words(int n, Word&& word, F&& f) {
+  auto fill = [&](auto& w) {
+    for (int i = 0; i < n; ++i) w.v[i] = word(i);
+    return f(w);
+  };
+  if (n <= 256) {
+    Words<256> w;
+    return fill(w);
+  }
+  if (n <= 1536) {
+    Words<1536> w;
+    return fill(w);
+  }
+  Words<kMaxWords> w;
+  return fill(w);
 }
 
 int ensure_buffer(pie_ctx* ctx, void** buf, size_t* cap, size_t need) {
@@ -234,12 +308,7 @@ void pie_plan_bind(pie_plan* plan, const PlanLayout& L, uint8_t* base) {
 int pie_launch_append(pie_ctx* ctx, const pie_plan* plan, const void* k_new, const void* v_new, cudaStream_t s) {
   if (plan->T == 0) return PIE_OK;
   const PoolGeom& g = ctx->geom;
-  auto log2i = [](int x) {
-    int l = 0;
-    while ((1 << l) < x) ++l;
-    return l;
-  };
-  const int chunk_shift = log2i(g.row_bytes >> 4), page_shift = log2i(g.page_size);   // (both powers of two: D 64 / 128, page size 8 / 16 / 32)
+  const int chunk_shift = log2_exact(g.row_bytes >> 4), page_shift = log2_exact(g.page_size);   // (both powers of two: D 64 / 128, page size 8 / 16 / 32)
   const int per_tok = (2 * g.n_kv_heads) << chunk_shift;
   int tok_shift = 0;   // tokens per block and step: as many as fit into 256 threads, a power of two
   while ((per_tok << (tok_shift + 1)) <= 256) ++tok_shift;
@@ -262,16 +331,23 @@ int pie_append_and_q(pie_ctx* ctx, const pie_plan* plan, const void* q, const vo
 }
 
 int pie_launch_copy(pie_ctx* ctx, int n, const int32_t* d_ops, cudaStream_t s) {
-  PIE_CUDA(ctx, pie_launch_pdl(copy_kernel, dim3(n, kCopySplit), dim3(256), 0, s, ctx->pool, d_ops, ctx->geom));
+  PIE_CUDA(ctx, pie_launch_pdl(plan_copy_kernel, dim3(n, kCopySplit), dim3(256), 0, s, ctx->pool, d_ops, ctx->geom,
+                               log2_exact(ctx->geom.row_bytes >> 4)));
   return PIE_OK;
 }
 
-int pie_launch_page_io(pie_ctx* ctx, int n, const int32_t* d_ids, void* K, void* V, bool write, cudaStream_t s) {
-  const PoolGeom& g = ctx->geom;
-  int64_t work = (int64_t)n * g.page_size * g.n_kv_heads * (g.row_bytes >> 4) * 2;
-  page_io_kernel<<<grid_for(work, 256, ctx->n_sms), 256, 0, s>>>(ctx->pool, d_ids, (uint8_t*)K, (uint8_t*)V, n,
-                                                                  write ? 1 : 0, g);
-  PIE_CUDA(ctx, cudaGetLastError());
+// copy_kvpage of up to kMaxWords / 3 operations
+template <int N>
+static int launch_copy_words(pie_ctx* ctx, int n, const Words<N>& w, cudaStream_t s) {
+  PIE_CUDA(ctx, pie_launch_pdl(copy_kernel<N>, dim3(n, kCopySplit), dim3(256), 0, s, ctx->pool, w, ctx->geom, log2_exact(ctx->geom.row_bytes >> 4)));
+  return PIE_OK;
+}
+
+// canonical K and V of n <= kMaxWords pages
+template <int N>
+static int launch_page_io(pie_ctx* ctx, int n, const Words<N>& w, void* K, void* V, bool write, cudaStream_t s) {
+  PIE_CUDA(ctx, pie_launch_pdl(page_io_kernel<N>, dim3(n, 2), dim3(256), 0, s, ctx->pool, w, (uint8_t*)K, (uint8_t*)V, write ? 1 : 0, ctx->geom,
+                               log2_exact(ctx->geom.row_bytes >> 4)));
   return PIE_OK;
 }
 
@@ -520,26 +596,28 @@ static int page_io(pie_ctx* ctx, int32_t n, const int32_t* ids, void* K, void* V
   cudaStream_t s = (cudaStream_t)stream;
   PIE_CUDA(ctx, cudaSetDevice(ctx->cfg.device));
   const size_t canon = (size_t)ctx->geom.page_size * ctx->geom.n_kv_heads * ctx->geom.row_bytes;  // K (or V) bytes per page
+  auto move = [&](int i0, int m, void* k, void* v) {   // pages i0 .. i0 + m (at most kMaxWords)
+    return with_words(m, [&](int i) { return ids[i0 + i]; }, [&](const auto& w) { return launch_page_io(ctx, m, w, k, v, write, s); });
+  };
   if (on_device) {
-    int rc = ensure_buffer(ctx, &ctx->d_stage, &ctx->stage_bytes, (size_t)n * 4);
-    if (rc) return rc;
-    PIE_CUDA(ctx, cudaMemcpyAsync(ctx->d_stage, ids, (size_t)n * 4, cudaMemcpyHostToDevice, s));
-    return pie_launch_page_io(ctx, n, (const int32_t*)ctx->d_stage, K, V, write, s);
+    for (int i0 = 0; i0 < n; i0 += kMaxWords) {
+      const int rc = move(i0, std::min(kMaxWords, n - i0), (uint8_t*)K + (size_t)i0 * canon, (uint8_t*)V + (size_t)i0 * canon);
+      if (rc) return rc;
+    }
+    return PIE_OK;
   }
-  const int chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)n, ((size_t)64 << 20) / canon));
-  size_t ids_bytes = ((size_t)chunk * 4 + 255) & ~(size_t)255;
-  int rc = ensure_buffer(ctx, &ctx->d_stage, &ctx->stage_bytes, ids_bytes + 2 * chunk * canon);
+  const int chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)std::min(n, kMaxWords), ((size_t)64 << 20) / canon));
+  int rc = ensure_buffer(ctx, &ctx->d_stage, &ctx->stage_bytes, 2 * chunk * canon);
   if (rc) return rc;
-  uint8_t* dK = (uint8_t*)ctx->d_stage + ids_bytes;
+  uint8_t* dK = (uint8_t*)ctx->d_stage;
   uint8_t* dV = dK + (size_t)chunk * canon;
   for (int i0 = 0; i0 < n; i0 += chunk) {
     int m = std::min(chunk, n - i0);
-    PIE_CUDA(ctx, cudaMemcpyAsync(ctx->d_stage, ids + i0, (size_t)m * 4, cudaMemcpyHostToDevice, s));
     if (write) {
       PIE_CUDA(ctx, cudaMemcpyAsync(dK, (const uint8_t*)K + (size_t)i0 * canon, (size_t)m * canon, cudaMemcpyHostToDevice, s));
       PIE_CUDA(ctx, cudaMemcpyAsync(dV, (const uint8_t*)V + (size_t)i0 * canon, (size_t)m * canon, cudaMemcpyHostToDevice, s));
     }
-    rc = pie_launch_page_io(ctx, m, (const int32_t*)ctx->d_stage, dK, dV, write, s);
+    rc = move(i0, m, dK, dV);
     if (rc) return rc;
     if (!write) {
       PIE_CUDA(ctx, cudaMemcpyAsync((uint8_t*)K + (size_t)i0 * canon, dK, (size_t)m * canon, cudaMemcpyDeviceToHost, s));
@@ -587,18 +665,21 @@ int pie_copy_kvpage(pie_ctx* ctx, int32_t n, const int32_t* src, const int32_t* 
   if (n == 0) return PIE_OK;
   cudaStream_t s = (cudaStream_t)stream;
   PIE_CUDA(ctx, cudaSetDevice(ctx->cfg.device));
-  std::vector<int32_t> ops((size_t)n * 5);
-  for (int k = 0; k < n; ++k) {
-    ops[k * 5 + 0] = src[k];
-    ops[k * 5 + 1] = dst[k];
-    ops[k * 5 + 2] = src_off[k];
-    ops[k * 5 + 3] = dst_off[k];
-    ops[k * 5 + 4] = ntok[k];
-  }
-  int rc = ensure_buffer(ctx, &ctx->d_stage, &ctx->stage_bytes, ops.size() * 4);
-  if (rc) return rc;
-  PIE_CUDA(ctx, cudaMemcpyAsync(ctx->d_stage, ops.data(), ops.size() * 4, cudaMemcpyHostToDevice, s));
-  return timed_launch(ctx, PIE_KERNEL_COPY, s, [&] { return pie_launch_copy(ctx, n, (const int32_t*)ctx->d_stage, s); });
+  const int most = kMaxWords / 3;
+  return timed_launch(ctx, PIE_KERNEL_COPY, s, [&] {
+    for (int k0 = 0; k0 < n; k0 += most) {
+      const int m = std::min(most, n - k0);
+      const int rc = with_words(
+          3 * m,
+          [&](int i) {
+            const int k = k0 + i / 3, f = i % 3;
+            return f == 0 ? src[k] : f == 1 ? dst[k] : src_off[k] | dst_off[k] << 8 | ntok[k] << 16;
+          },
+          [&](const auto& w) { return launch_copy_words(ctx, m, w, s); });
+      if (rc) return rc;
+    }
+    return (int)PIE_OK;
+  });
 }
 
 // Plans are recycled: pie_plan_destroy parks up to kParkedPlans objects in the context, with their

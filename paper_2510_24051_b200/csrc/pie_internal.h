@@ -280,8 +280,7 @@ int pie_launch_rope(pie_ctx* ctx, const pie_plan* plan, const void* q, const voi
 // append (plain or RoPE) and the Q the attention kernels must read
 int pie_append_and_q(pie_ctx* ctx, const pie_plan* plan, const void* q, const void* k_new, const void* v_new, cudaStream_t s,
                      const void** q_eff);
-int pie_launch_copy(pie_ctx* ctx, int n, const int32_t* d_ops, cudaStream_t s);
-int pie_launch_page_io(pie_ctx* ctx, int n, const int32_t* d_ids, void* K, void* V, bool write, cudaStream_t s);
+int pie_launch_copy(pie_ctx* ctx, int n, const int32_t* d_ops, cudaStream_t s);   // operations of a plan, in device memory
 int pie_launch_simple(pie_ctx* ctx, const pie_plan* plan, const void* q, void* out, float* lse, cudaStream_t s);
 int pie_launch_split(pie_ctx* ctx, const pie_plan* plan, const void* q, const void* k_new, const void* v_new, void* out,
                      float* lse, cudaStream_t s);
@@ -337,8 +336,12 @@ void pie_free_pages(pie_ctx* ctx, const std::vector<int32_t>& ids);
 __device__ __forceinline__ void pie_pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pie_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-template <typename... KArgs, typename... Args>
-cudaError_t pie_launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+template <typename T>
+struct PieSame { typedef T type; };   // (arguments convert to the kernel's parameter types instead of taking part in deduction)
+
+template <typename... KArgs>
+cudaError_t pie_launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                           const typename PieSame<KArgs>::type&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -349,6 +352,7 @@ cudaError_t pie_launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+  void* ptrs[] = {const_cast<void*>(static_cast<const void*>(&args))...};   // (by address: parameter blocks reach 32 KB)
+  return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kern), ptrs);
 }
 #endif
