@@ -373,7 +373,9 @@ int pie_sched_next_batch(pie_sched* s, int32_t* out_type, int32_t cap, int64_t* 
  *                      By default a group whose pieces are the last work of their warps leaves
  *                      them in the warps' idle staging buffers in shared memory.  Bit 2: one kv head per
  *                      decode unit.  By default, with 64-wide heads and pages of 8 or 16 tokens, a
- *                      unit is a pair of adjacent kv heads (one copy of twice the size per page). */
+ *                      unit is a pair of adjacent kv heads (one copy of twice the size per page).  Bit 4: no
+ *                      clusters.  By default every unit of a launch of few or short units is owned by a
+ *                      cluster of thread blocks that merges its pieces through (distributed) shared memory. */
 enum { PIE_OPT_SPLIT_SMS = 0, PIE_OPT_TILE_SMS = 1, PIE_OPT_OVERLAP = 2, PIE_OPT_NO_FUSION = 3, PIE_NUM_OPTIONS = 4 };
 int pie_set_option(pie_ctx* ctx, int option, int value);
 

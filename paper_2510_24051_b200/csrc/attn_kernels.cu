@@ -752,6 +752,219 @@ __global__ void __launch_bounds__(NW * 32, 1) attn_split_kernel(const AttnParams
   }
 }
 
+// ------------------------------------------------------------------------------ short units: a cluster or a block per unit
+// Decode launches of a few requests, or of short contexts, are a chain of latencies, not a stream: the two-level merge of
+// attn_split_kernel (a block's pieces through shared memory and a spinning warp; the blocks' partials through L2 with a
+// device-wide fence, an atomic and two dependent reads) was 5 - 6 us of a 17 - 21 us launch of four requests.  Here every
+// unit belongs to ONE cluster of up to 8 thread blocks: each warp takes one contiguous piece of the unit's visits, the
+// pieces of a block meet in shared memory behind a block barrier - every thread combines one float4 of the rows - and the
+// blocks' partials in distributed shared memory behind a cluster barrier, where every block finishes its share of the
+// rows.  No partial goes through L2 and nobody spins.  Sources are combined in page order, so results do not depend on timing.
+// With more units than clusters a unit has one block of 8, 4, 2 or 1 warps to itself, several blocks to an SM.
+// The planner (pick_cluster, partition_cluster) chooses all that; the items carry the same piece fields as a two-level launch.
+template <int D, int P, int NW, int DEPTH, int HP>
+struct ClusterCfg {
+  static constexpr int PPV = P == 8 ? 2 : 1;
+  static constexpr int PAGE = 2 * P * D * 2;
+  static constexpr int VP = HP * PAGE;
+  static constexpr int STAGE = PPV * VP;
+  static constexpr int PART = 16 * D + 16;   // floats of a partial: 16 rows, 16 LSEs
+  static constexpr int BAR_OFF = NW * DEPTH * STAGE;
+  static constexpr int META_OFF = BAR_OFF + NW * DEPTH * 8;                 // per stage and page: logical page | flag, physical page
+  static constexpr int PART_OFF = (META_OFF + NW * DEPTH * PPV * 8 + 15) & ~15;
+  static constexpr bool FULL = NW == (P == 32 && D == 128 ? 4 : 8);         // (smaller blocks own their unit alone: no block partial)
+  static constexpr int SMEM = PART_OFF + (FULL ? PART * 4 : 0);
+  static_assert(PART * 4 <= DEPTH * STAGE, "a warp's partial fits over its idle ring");
+};
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float4 cluster_ld4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ float cluster_ld(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+  return v;
+}
+
+// LSE-weighted combination of one float4 of a row over `n` sources (n <= 8): load(c, lse, vec).
+template <class Load>
+__device__ __forceinline__ void combine4(int n, Load&& load, float4& out, float& lse_out) {
+  float l[8];
+  float4 v[8];
+  float M = kNegInf;
+#pragma unroll
+  for (int c = 0; c < 8; ++c)
+    if (c < n) {
+      load(c, l[c], v[c]);
+      M = fmaxf(M, l[c]);
+    }
+  float Z = 0.f;
+  float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int c = 0; c < 8; ++c)
+    if (c < n) {
+      const float w = M == kNegInf ? 0.f : __expf(l[c] - M);   // exp(-inf) = 0
+      Z += w;
+      a.x += w * v[c].x, a.y += w * v[c].y, a.z += w * v[c].z, a.w += w * v[c].w;
+    }
+  const float inv = Z > 0.f ? 1.f / Z : 0.f;
+  out = make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv);
+  lse_out = Z > 0.f ? M + logf(Z) : kNegInf;
+}
+
+template <int D, int P, int NW, int DEPTH, int HP>
+__global__ void __launch_bounds__(NW * 32, 1) decode_cluster_kernel(const AttnParams p, const int cluster_size) {
+  using C = ClusterCfg<D, P, NW, DEPTH, HP>;
+  constexpr int PPV = C::PPV;
+  static_assert(NW <= 8, "a block's pieces are combined from registers");
+  extern __shared__ __align__(1024) uint8_t smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint8_t* stages = smem + warp * DEPTH * C::STAGE;
+  const uint32_t full_bar = smem_u32(smem + C::BAR_OFF) + warp * DEPTH * 8;
+  volatile uint32_t* meta = reinterpret_cast<uint32_t*>(smem + C::META_OFF) + warp * DEPTH * PPV * 2;
+  float* part = reinterpret_cast<float*>(smem + C::PART_OFF);
+  if (!p.late_trigger) pie_pdl_launch_dependents();
+  if (lane == 0) {
+    for (int s = 0; s < DEPTH; ++s) mbar_init(full_bar + 8 * s, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncwarp();
+
+  // Plan arrays (not written by the kernels in front): the cluster's pieces, one per warp from its first warp on, this
+  // warp's piece and its first page records - all before the wait.
+  const int c0 = (int)blockIdx.x / cluster_size * cluster_size, rank = (int)blockIdx.x - c0;
+  const int first = p.cta_ptr[c0 * NW], n_pieces = p.cta_ptr[(c0 + cluster_size) * NW] - first;
+  const int my_piece = rank * NW + warp;
+  const bool have = my_piece < n_pieces;
+  const PieItem item = p.items[first + (have ? my_piece : 0)];
+  const int n_pages = have ? item.page_end - item.page_begin : 0, n_visits = (n_pages + PPV - 1) / PPV;
+  int2 pre[DEPTH][PPV];
+#pragma unroll
+  for (int i = 0; i < DEPTH; ++i)
+#pragma unroll
+    for (int j = 0; j < PPV; ++j) {
+      pre[i][j] = make_int2(0, 0);
+      if (i * PPV + j < n_pages) pre[i][j] = __ldg(&p.kept[item.page_begin + i * PPV + j]);
+    }
+  auto issue = [&](int n, const int2* rec) {   // visit n of the piece (lane 0)
+    const uint32_t s = n % DEPTH;
+    const int cnt = min(PPV, n_pages - n * PPV);
+#pragma unroll
+    for (int i = 0; i < PPV; ++i) {
+      meta[(s * PPV + i) * 2] = i < cnt ? (uint32_t)rec[i].y : PIE_NO_PAGE;
+      meta[(s * PPV + i) * 2 + 1] = (uint32_t)rec[i].x;
+    }
+    mbar_expect_tx(full_bar + 8 * s, cnt * C::VP);
+#pragma unroll
+    for (int i = 0; i < PPV; ++i)
+      if (i < cnt)
+        bulk_g2s(smem_u32(stages + s * C::STAGE + i * C::VP), p.pool + ((int64_t)rec[i].x * p.n_kv_heads + item.kv_head * HP) * C::PAGE, C::VP,
+                 full_bar + 8 * s);
+  };
+  pie_pdl_wait();
+  if (have) {
+#pragma unroll
+    for (int i = 0; i < DEPTH; ++i)
+      if (i < n_visits && lane == 0) issue(i, pre[i]);
+    PieReq rq;
+    rq.q_start = item.q_start, rq.q_len = item.q_len, rq.kv_len = item.kv_len, rq.kept_start = 0, rq.kept_count = 0;
+    rq.mask_row_words = item.mask_row_words, rq.mask_word_off = item.mask_word_off;
+    rq.last_logical = item.last_logical, rq.last_page_len = item.last_page_len;
+    // (fused append: as in attn_split_kernel, the piece that ends with the request's last page writes the new row)
+    constexpr int CH = D * 2 / 16;
+    const bool do_append = (item.flags & PIE_ITEM_APPEND) != 0;
+    const int a_head = lane / (2 * CH), a_v = (lane / CH) & 1;
+    uint4 new_chunk = make_uint4(0, 0, 0, 0);
+    if (do_append && lane < 2 * CH * HP)
+      new_chunk = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(a_v ? p.v_new : p.k_new) +
+                                                       ((int64_t)item.q_start * p.n_kv_heads + item.kv_head * HP + a_head) * (D * 2)) + (lane % CH));
+    RowState<D> st;
+    rows_init<D>(st, p, item, rq, item.row0, lane);
+    for (int n = 0; n < n_visits; ++n) {
+      const uint32_t s = n % DEPTH, ph = (n / DEPTH) & 1;
+      int2 rec_next[PPV];
+      const bool refill = n + DEPTH < n_visits;
+#pragma unroll
+      for (int i = 0; i < PPV; ++i) {
+        rec_next[i] = make_int2(0, 0);
+        if (refill && (n + DEPTH) * PPV + i < n_pages) rec_next[i] = __ldg(&p.kept[item.page_begin + (n + DEPTH) * PPV + i]);
+      }
+      mbar_wait(full_bar + 8 * s, ph, p.status);
+      uint32_t lpf[PPV];
+#pragma unroll
+      for (int i = 0; i < PPV; ++i) {
+        lpf[i] = meta[(s * PPV + i) * 2];
+        if (do_append && lpf[i] != PIE_NO_PAGE && (int)(lpf[i] & ~PIE_KEPT_NEEDS_MASK) == item.last_logical) {
+          if (lane < 2 * CH * HP) {
+            const int off = a_head * C::PAGE + (a_v ? C::PAGE / 2 : 0) + pie_chunk_offset(P * 128, item.last_page_len - 1, lane % CH);
+            *reinterpret_cast<uint4*>(stages + s * C::STAGE + i * C::VP + off) = new_chunk;
+            const int phys = (int)meta[(s * PPV + i) * 2 + 1];
+            *reinterpret_cast<uint4*>(const_cast<uint8_t*>(p.pool) + ((int64_t)phys * p.n_kv_heads + item.kv_head * HP) * C::PAGE + off) = new_chunk;
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+        }
+      }
+      visit_compute<D, P, PPV, HP>(st, stages + s * C::STAGE, rq, lpf, p.scale_log2, lane);
+      __syncwarp();
+      if (refill && lane == 0) issue(n + DEPTH, rec_next);
+    }
+    rows_store_smem<D>(st, reinterpret_cast<float*>(stages), lane);
+  }
+  __syncthreads();
+
+  // ---- the block's pieces into one partial, then the cluster's partials into the rows
+  const int in_block = min(NW, n_pieces - rank * NW), n_blocks = (n_pieces + NW - 1) / NW;
+  const int n_vec = item.nrows * (D / 4);   // float4s of the unit's rows
+  auto finish = [&](int e, const float4& a, float lse) {   // (every piece of the unit has the same rows)
+    const int row = e / (D / 4), gr = item.row0 + row;
+    const int64_t oi = (int64_t)(item.q_start + gr / p.G) * p.n_q_heads + item.kv_head * p.G + gr % p.G;
+    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + oi * D + (e % (D / 4)) * 4) = make_uint2(pack_bf16(a.x, a.y), pack_bf16(a.z, a.w));
+    if (e % (D / 4) == 0) p.lse[oi] = lse;
+  };
+  for (int e = threadIdx.x; e < n_vec && in_block > 0; e += NW * 32) {
+    const int row = e / (D / 4);
+    float4 a;
+    float lse;
+    combine4(in_block, [&](int c, float& l, float4& v) {
+      const float* src = reinterpret_cast<const float*>(smem + c * DEPTH * C::STAGE);
+      l = src[16 * D + row];
+      v = *reinterpret_cast<const float4*>(src + e * 4);
+    }, a, lse);
+    if (n_blocks == 1) {
+      finish(e, a, lse);
+    } else {
+      *reinterpret_cast<float4*>(part + e * 4) = a;
+      if (e % (D / 4) == 0) part[16 * D + row] = lse;
+    }
+  }
+  if (n_blocks <= 1) return;   // (uniform over the cluster)
+  cluster_arrive();
+  cluster_wait();
+  for (int e = rank + cluster_size * (int)threadIdx.x; e < n_vec; e += cluster_size * NW * 32) {
+    const int row = e / (D / 4);
+    float4 a;
+    float lse;
+    combine4(n_blocks, [&](int c, float& l, float4& v) {
+      const uint32_t src = cluster_map(smem_u32(part), (uint32_t)c);
+      l = cluster_ld(src + (16 * D + row) * 4);
+      v = cluster_ld4(src + e * 16);
+    }, a, lse);
+    finish(e, a, lse);
+  }
+  cluster_arrive();   // no block leaves while another may still read its partial
+  cluster_wait();
+}
+
 // ------------------------------------------------------------------------------ row-tile kernel
 // Prefill chunks and token trees: NW consumer warps own 16 query rows each and all walk the same
 // page stream, which a producer warp keeps filled through a ring of full / empty barriers.
@@ -1140,6 +1353,58 @@ int launch_split(pie_ctx* ctx, const AttnParams& p, int n_items, int n_warps, cu
   return PIE_OK;
 }
 
+// The cluster kernel of the context's shape with blocks of `warps` warps: every caller names the instantiation through this.
+template <class F>
+int with_cluster_kernel(const pie_ctx* ctx, int hp, int warps, F&& f) {
+  const int D = ctx->cfg.head_dim, P = ctx->cfg.page_size;
+#define PIE_CLUSTER1(DD, PP, NW, DEPTH, HP) \
+  if (warps == NW) return f(decode_cluster_kernel<DD, PP, NW, DEPTH, HP>, ClusterCfg<DD, PP, NW, DEPTH, HP>::SMEM)
+#define PIE_CLUSTER(DD, PP, NW, DEPTH, HP)             \
+  if (D == DD && P == PP && hp == HP) {                \
+    PIE_CLUSTER1(DD, PP, NW, DEPTH, HP);               \
+    PIE_CLUSTER1(DD, PP, NW / 2, DEPTH, HP);           \
+    PIE_CLUSTER1(DD, PP, NW / 4, DEPTH, HP);           \
+    if (NW == 8) PIE_CLUSTER1(DD, PP, 1, DEPTH, HP);   \
+  }
+  PIE_CLUSTER(64, 16, 8, 3, 2)
+  PIE_CLUSTER(64, 8, 8, 3, 2)
+  PIE_CLUSTER(64, 8, 8, 4, 1)
+  PIE_CLUSTER(128, 8, 8, 3, 1)
+  PIE_CLUSTER(64, 16, 8, 4, 1)
+  PIE_CLUSTER(128, 16, 8, 3, 1)
+  PIE_CLUSTER(64, 32, 8, 3, 1)
+  PIE_CLUSTER(128, 32, 4, 3, 1)
+#undef PIE_CLUSTER
+#undef PIE_CLUSTER1
+  return PIE_ERR_UNSUPPORTED;
+}
+
+int launch_cluster(pie_ctx* ctx, const AttnParams& p, int hp, int warps, int cluster_size, int blocks, cudaStream_t s) {
+  return with_cluster_kernel(ctx, hp, warps, [&](auto kern, int smem) -> int {
+    bool& configured = ctx->cluster_configured[hp - 1][warps == 8 ? 3 : warps >> 1];
+    if (!configured) {
+      PIE_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      configured = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)warps * 32);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster_size;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    PIE_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, p, cluster_size));
+    return PIE_OK;
+  });
+}
+
 template <int D, int P, int NW>
 int launch_tiles(pie_ctx* ctx, const AttnParams& p, int grid, cudaStream_t s) {
   constexpr int NSTAGES = (128 * 1024) / (2 * P * D * 2);
@@ -1168,6 +1433,36 @@ bool pie_split_pair_supported(const pie_ctx* ctx) {
          2 * ctx->G <= 16;
 }
 
+// Clusters of 2 / 4 / 8 full blocks of the cluster kernel that are resident at once (0: the device cannot place them).  Asked
+// once per context and unit width; a host-only context assumes a whole B200.
+int pie_split_max_clusters(pie_ctx* ctx, int hp, int cluster_size) {
+  if (ctx->host_only) return cluster_size == 8 ? 16 : 144 / cluster_size;
+  int& known = ctx->max_clusters[hp - 1][cluster_size == 2 ? 0 : cluster_size == 4 ? 1 : 2];
+  if (known >= 0) return known;
+  known = 0;
+  const int warps = pie_split_warps_per_block(ctx);
+  with_cluster_kernel(ctx, hp, warps, [&](auto kern, int smem) -> int {
+    PIE_CUDA(ctx, cudaSetDevice(ctx->cfg.device));
+    PIE_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)cluster_size);
+    cfg.blockDim = dim3((unsigned)warps * 32);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cluster_size;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess) known = n;
+    else cudaGetLastError();
+    return PIE_OK;
+  });
+  return known;
+}
+
 // Warps per block of the split-KV kernel (the planner sizes its shares with this).
 int pie_split_warps_per_block(const pie_ctx* ctx) {
   return (ctx->cfg.page_size == 32 && ctx->cfg.head_dim == 128) ? 4 : 8;
@@ -1180,6 +1475,8 @@ int pie_launch_split(pie_ctx* ctx, const pie_plan* plan, const void* q, const vo
   p.v_new = v_new;
   const int D = ctx->cfg.head_dim, P = ctx->cfg.page_size, n = plan->split.grid, ni = (int)plan->split.items.size();
   if (ctx->cfg.dtype == PIE_DTYPE_F32) return pie_launch_f32(ctx, p, n, plan->split.slot_rows, false, s);
+  if (plan->split.cluster > 0)
+    return launch_cluster(ctx, p, plan->split.heads_per_unit, plan->split.cluster_warps, plan->split.cluster, n / plan->split.cluster_warps, s);
   // ring depth: 128 - 192 KB of copies in flight per SM (measured on the 64-request decode batch with 4 KB stages:
   // depths 3 and 4 run 1.5 % faster than 5 and 6 - a deeper ring only lengthens the queue in front of every copy)
   if (plan->split.heads_per_unit == 2) {   // units of two adjacent kv heads: copies of 8 KB instead of 4 KB (of 4 KB instead of 2 KB)

@@ -114,6 +114,8 @@ struct PieLaunchList {           // one tile-kernel launch (split-KV decode, or 
   int32_t slot_rows = 0;
   int32_t n_static = 0;          // split-KV: items [n_static, size) are taken from the work counter
   bool grid_merge = false;       // split-KV: cut units are merged inside the kernel by their last piece (one counter per slot behind d_work_ctr)
+  int32_t cluster = 0;           // split-KV: blocks of the cluster that owns a unit (decode_cluster_kernel); 0: attn_split_kernel
+  int32_t cluster_warps = 0;     // ... and warps of each of these blocks
   int32_t heads_per_unit = 1;    // split-KV: 2 = every item covers kv heads 2 kv_head and 2 kv_head + 1 (rows of the first, then of the second)
   // device copies
   PieItem* d_items = nullptr;
@@ -215,6 +217,8 @@ struct pie_ctx {
   struct HeldPages { cudaEvent_t done; std::vector<int32_t> pages; };
   std::vector<HeldPages> held_pages;
   std::vector<cudaEvent_t> held_events;   // recycled events of held_pages
+  bool cluster_configured[2][4] = {};   // (units of one / of two kv heads; blocks of 1, 2, 4, 8 warps)
+  int max_clusters[2][3] = {{-1, -1, -1}, {-1, -1, -1}};   // pie_split_max_clusters: of 2 / 4 / 8 blocks; -1: not asked yet
   bool f32_configured[3] = {false, false, false};   // (items of <= 4, <= 16, 64 rows)
   bool tc_configured = false, split_configured = false, split_pair_configured = false, tile_configured = false, nd_configured[6] = {false, false, false, false, false, false};   // kernel attributes set for this context's device
   // The block-local work list of the latest decode batch.  Consecutive steps of a serving loop bring the same
@@ -289,6 +293,7 @@ int pie_launch_merge(pie_ctx* ctx, const pie_plan* plan, const PieLaunchList& ll
 bool pie_split_supported(const pie_ctx* ctx);
 bool pie_split_pair_supported(const pie_ctx* ctx);   // ... with units of two adjacent kv heads
 int pie_split_warps_per_block(const pie_ctx* ctx);
+int pie_split_max_clusters(pie_ctx* ctx, int hp, int cluster_size);
 bool pie_tc_supported(const pie_ctx* ctx);
 // fp32 pools (attn_f32_kernel.cu): one launch list; tiles: items of 64 rows, else of at most max_rows <= 16
 int pie_launch_f32(pie_ctx* ctx, const AttnParams& p, int grid, int max_rows, bool tiles, cudaStream_t s);

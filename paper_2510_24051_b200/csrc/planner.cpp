@@ -539,6 +539,47 @@ bool partition_local(const std::vector<Unit>& units, int ctas_max, int NW, int m
   return true;
 }
 
+// Split-KV decode, short units: every unit gets a cluster of `cluster` blocks of NW warps to itself and is cut into one
+// piece of whole visits (`ppv` pages) per warp, from the cluster's first warp on.  The pieces carry the fields of a
+// two-level merge (PIE_ITEM_LOCAL_* inside a block, PIE_ITEM_GRID_* between the unit's blocks).
+void partition_cluster(const std::vector<Unit>& units, int cluster, int NW, int ppv, int slot_rows, PieLaunchList& ll) {
+  ll.items.clear();
+  ll.merges.clear();
+  ll.cta_ptr.clear();
+  ll.slot_rows = slot_rows;
+  ll.n_slots = 0;
+  ll.n_static = 0;
+  ll.cluster = cluster;
+  ll.cluster_warps = NW;
+  const int width = cluster * NW;
+  ll.grid = (int)units.size() * width;
+  ll.items.reserve((size_t)ll.grid);
+  ll.cta_ptr.reserve((size_t)ll.grid + 1);
+  ll.cta_ptr.push_back(0);
+  for (const Unit& u : units) {
+    const int n = u.page_end - u.page_begin, visits = (n + ppv - 1) / ppv;
+    const int np = std::max(1, std::min(visits, width)), nb = (np + NW - 1) / NW;
+    for (int k = 0; k < np; ++k) {
+      PieItem it = make_item(u, u.page_begin + std::min(n, (int)((int64_t)visits * k / np) * ppv),
+                             u.page_begin + std::min(n, (int)((int64_t)visits * (k + 1) / np) * ppv));
+      if (np > 1) {
+        const int kb = k / NW, in_block = std::min(NW, np - kb * NW);
+        it.partial_slot = ll.n_slots + k;
+        if (in_block > 1) it.flags |= PIE_ITEM_LOCAL_PIECE | PIE_ITEM_LOCAL_BITS(0, in_block);
+        if (k % NW == 0) {
+          if (in_block > 1) it.flags |= PIE_ITEM_LOCAL_MERGER;
+          if (nb > 1) it.flags |= PIE_ITEM_GRID_PIECE | PIE_ITEM_GRID_BITS(nb, kb, NW);
+        }
+      }
+      ll.items.push_back(it);
+      ll.cta_ptr.push_back((int32_t)ll.items.size());
+    }
+    if (np > 1) ll.n_slots += np;
+    for (int k = np; k < width; ++k) ll.cta_ptr.push_back((int32_t)ll.items.size());   // warps without a piece
+  }
+  ll.n_static = (int32_t)ll.items.size();
+}
+
 // Block-local merge groups (PIE_ITEM_LOCAL_*) all of whose pieces are the last items of their warps leave
 // their partials in shared memory: mark them.  `ll.cta_ptr` holds one item range per warp; the pieces of a
 // group are consecutive items, the merging one first.
@@ -643,6 +684,37 @@ void chunk_units(const std::vector<Unit>& units, int n_warps, PieLaunchList& ll)
 }  // namespace
 
 static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan);
+
+// Should every unit of a decode launch get a cluster of blocks - or a block - to itself (partition_cluster)?  `blocks` of
+// `warps` warps: the most for which the whole launch is resident at once, no more than the longest unit has use for.
+// Otherwise (false) shares over all warps of the chip.
+static bool pick_cluster(pie_ctx* ctx, const std::vector<Unit>& units, bool plain, int64_t W, int sms, int hp, bool side_by_side, int* blocks,
+                         int* warps) {
+  if (units.empty() || !plain || side_by_side || sms != ctx->n_sms || (ctx->options[PIE_OPT_NO_FUSION] & (2 | 8 | 16))) return false;
+  const int NW = pie_split_warps_per_block(ctx), ppv = ctx->cfg.page_size == 8 ? 2 : 1, n = (int)units.size();
+  int longest_pages = 0;
+  for (const Unit& u : units) longest_pages = std::max(longest_pages, u.page_end - u.page_begin);
+  const int longest = (longest_pages + ppv - 1) / ppv;
+  int c = 0, w = 1;
+  for (int k = 1; k <= NW && n <= sms * (NW / k); k *= 2) {   // blocks of k warps: NW / k of them fit an SM
+    c = 1, w = k;
+    if (k >= longest) break;
+  }
+  if (c == 0) return false;
+  for (int k = 2; w == NW && c * w < longest && k <= 8 && n <= pie_split_max_clusters(ctx, hp, k); k *= 2) c = k;
+  // The launch lasts as long as its longest piece, the alternative as its equal shares and its merges: those cost it about
+  // 11 visits' time when units are cut across blocks, 5 when they are dealt to blocks whole (the test is the one of
+  // partition_local).  Measured on 1 - 200 requests of 20 - 8,000 tokens (32 / 8 heads of 64 and of 128, 16 / 2, 12 / 12;
+  // 8-, 16- and 32-token pages), in brackets the alternative, us per launch: 1 x 2,000 tokens 6.3 (19.5), 4 x 150 5.2 (11.5),
+  // 4 x 2,000 8.0 (19.5), 4 x 8,000 18.0 (22.6), 12 x 2,000 12.9 (22.6), 24 x 600 8.1 (12.3), 96 x 150 8.2 (12.9),
+  // 200 x 150 14.7 (17.5); no size it accepts was slower.
+  const int64_t piece = (longest + c * w - 1) / (c * w), share = std::max<int64_t>(4, W / ppv / ((int64_t)sms * NW));
+  const bool cut = (int64_t)longest_pages * sms * 100 > W * 108 && longest_pages > W / sms + 100;
+  if (piece > share + share / 8 + (cut ? 11 : 5)) return false;
+  *blocks = c;
+  *warps = w;
+  return true;
+}
 
 // Scratch pages a plan holds for requests without output KvPages go back to the free list.
 void pie_free_pages(pie_ctx* ctx, const std::vector<int32_t>& ids) {
@@ -1348,6 +1420,7 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
     }
     plan->split.heads_per_unit = hp;
     plan->split.grid_merge = false;
+    plan->split.cluster = 0;
     const double kv_bytes = (double)W * hp * 2.0 * P * cfg.head_dim * (cfg.dtype == PIE_DTYPE_BF16 ? 2.0 : 4.0);
     const bool long_launch = kv_bytes * ctx->n_sms >= 1.6e9 * split_sms;   // (fewer SMs: the same bytes take longer)
     bool plain_units = true;
@@ -1357,6 +1430,8 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
       // (a block takes a 16-token page in about 0.1 us, the launch 4 - 5 us)
       partition(split_units, split_sms * pie_f32_blocks_per_sm(ctx, false), 16, max_rows, true, plan->split, nullptr, 45);
       plan->split.n_static = (int32_t)plan->split.items.size();
+    } else if (int c_blocks = 0, c_warps = 0; pick_cluster(ctx, split_units, plain_units, W, split_sms, hp, plan->overlap, &c_blocks, &c_warps)) {
+      partition_cluster(split_units, c_blocks, c_warps, P == 8 ? 2 : 1, max_rows, plan->split);
     } else if (long_launch || (W >= (int64_t)200 * n_warps && !plain_units)) {
       chunk_units(split_units, n_warps, plan->split);
     } else {
