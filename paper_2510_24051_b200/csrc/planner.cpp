@@ -702,15 +702,21 @@ static bool pick_cluster(pie_ctx* ctx, const std::vector<Unit>& units, bool plai
   }
   if (c == 0) return false;
   for (int k = 2; w == NW && c * w < longest && k <= 8 && n <= pie_split_max_clusters(ctx, hp, k); k *= 2) c = k;
-  // The launch lasts as long as its longest piece, the alternative as its equal shares and its merges: those cost it about
-  // 11 visits' time when units are cut across blocks, 5 when they are dealt to blocks whole (the test is the one of
-  // partition_local).  Measured on 1 - 200 requests of 20 - 8,000 tokens (32 / 8 heads of 64 and of 128, 16 / 2, 12 / 12;
-  // 8-, 16- and 32-token pages), in brackets the alternative, us per launch: 1 x 2,000 tokens 6.3 (19.5), 4 x 150 5.2 (11.5),
-  // 4 x 2,000 8.0 (19.5), 4 x 8,000 18.0 (22.6), 12 x 2,000 12.9 (22.6), 24 x 600 8.1 (12.3), 96 x 150 8.2 (12.9),
-  // 200 x 150 14.7 (17.5); no size it accepts was slower.
-  const int64_t piece = (longest + c * w - 1) / (c * w), share = std::max<int64_t>(4, W / ppv / ((int64_t)sms * NW));
+  // Estimates in us.  Here: 4.5 to start and merge, then the longest piece at the rate of a warp that has the memory system
+  // to itself, or the bytes at the chip's rate and half the time by which the longest piece outlasts an average one.  The
+  // alternative: the bytes, 11 to start and merge, and 4.5 more for the two-level merge of units cut across blocks (the
+  // test is the one of partition_local; behind more than 12 us of bytes that merge is hidden).  Measured on 1 - 200
+  // requests of 20 - 8,000 tokens (32 / 8 heads of 64 and of 128, 16 / 2, 12 / 12; 8-, 16- and 32-token pages), in
+  // brackets the alternative, us per launch: 1 x 2,000 tokens 6.3 (19.5), 4 x 2,000 8.0 (19.5), 4 x 8,000 18.0 (22.6),
+  // 12 x 2,000 12.9 (22.6), 24 x 600 8.1 (12.3), 48 x 2,000 31.5 (34.3), 200 x 600 38.8 (40.9); where lengths differ more
+  // it loses and is not taken: 48 requests of 100 - 2,000 tokens 29.5 (26.3).
+  const double visit_bytes = (double)ppv * hp * 4.0 * ctx->cfg.page_size * ctx->cfg.head_dim;
+  const double t_visit = ppv == 2 ? 1.08 : visit_bytes > 8192 ? 1.05 : 0.83;   // (two copies per visit; 16 KB visits)
+  const double t_bytes = (double)W / ppv * visit_bytes / 6.4e6;
+  const double piece = (double)((longest + c * w - 1) / (c * w)), mean = (double)W / ppv / ((double)n * c * w);
+  const double t_here = 4.5 + std::max(piece * t_visit, t_bytes + 0.5 * t_visit * std::max(0.0, piece - mean));
   const bool cut = (int64_t)longest_pages * sms * 100 > W * 108 && longest_pages > W / sms + 100;
-  if (piece > share + share / 8 + (cut ? 11 : 5)) return false;
+  if (t_here + 2.0 > t_bytes + (cut && t_bytes < 12 ? 15.5 : 11.0)) return false;
   *blocks = c;
   *warps = w;
   return true;
