@@ -222,7 +222,8 @@ PieItem make_item(const Unit& u, int32_t page_begin, int32_t page_end) {
 //  * Otherwise: contiguous equal shares; a unit cut by a share boundary becomes several items
 //    whose fp32 partials are merged.
 void partition(const std::vector<Unit>& units, int grid_max, int min_pages_per_cta, int slot_rows,
-               bool allow_whole_units, PieLaunchList& ll, UnitSlots* slots_out = nullptr, int slack_pages = 200) {
+               bool allow_whole_units, PieLaunchList& ll, UnitSlots* slots_out = nullptr, int slack_pages = 200,
+               double slack_per_piece = 0.0) {
   if (slots_out) slots_out->assign(units.size(), std::make_pair(-1, 0));
   ll.items.clear();
   ll.merges.clear();
@@ -237,15 +238,16 @@ void partition(const std::vector<Unit>& units, int grid_max, int min_pages_per_c
     W += u.page_end - u.page_begin;
     max_unit = std::max<int64_t>(max_unit, u.page_end - u.page_begin);
   }
-  const int grid = (int)std::min<int64_t>(grid_max, std::max<int64_t>(1, W / std::max(1, min_pages_per_cta)));
-  ll.grid = grid;
+  const int grid_cut = (int)std::min<int64_t>(grid_max, std::max<int64_t>(1, W / std::max(1, min_pages_per_cta)));
+  const int64_t slack = slack_pages + (int64_t)(slack_per_piece * (double)(units.size() + grid_cut));
+  int grid = std::min(grid_max, (int)units.size());   // (whole units: every one may have a CTA to itself, however short it is)
 
   // Whole units also when there are only a few per CTA (or fewer units than CTAs), as long as dealing them out
-  // (largest first then) leaves the fullest CTA within 12 % of the average or within `slack_pages` page visits (200:
-  // ~45 us of a row-tile CTA) of it: a cut unit costs fp32 partials of up to 256 rows, more and shorter items and the merge
-  // launch, which on a short launch is more than that imbalance (8 prefill chunks of 512 tokens: 137 -> 78 us;
-  // one prompt of 2,048 tokens: 90 -> 46 us although only 64 of 148 CTAs get a unit).
+  // (largest first then) leaves the fullest CTA within 12 % of the average share of a cut list or within `slack` page visits
+  // of it: a cut unit costs fp32 partials of up to 256 rows, more and shorter items and the merge launch, all in all
+  // `slack_pages` page visits' time and `slack_per_piece` more for every piece.
   const bool many_small = (int64_t)units.size() >= 4 * (int64_t)grid && max_unit * 8 <= W / grid;
+  ll.grid = grid;
   const bool few_whole = !many_small && allow_whole_units && W > 0;
   if (allow_whole_units && (many_small || few_whole)) {
     // least-loaded-first list scheduling (binary heap keyed on (load, cta)), then a counting sort
@@ -272,7 +274,7 @@ void partition(const std::vector<Unit>& units, int grid_max, int min_pages_per_c
       max_load = std::max(max_load, top.first);
       std::push_heap(heap.begin(), heap.end(), cmp);
     }
-    if (few_whole && max_load * grid * 100 > W * 112 && max_load > W / grid + slack_pages) goto contiguous;   // too uneven: cut the units instead
+    if (few_whole && max_load * grid_cut * 100 > W * 112 && max_load > W / grid_cut + slack) goto contiguous;   // too uneven: cut the units instead
     for (int c = 0; c < grid; ++c) ll.cta_ptr[c + 1] += ll.cta_ptr[c];
     std::vector<int32_t> fill(ll.cta_ptr.begin(), ll.cta_ptr.end() - 1);
     ll.items.resize(units.size());
@@ -291,6 +293,7 @@ void partition(const std::vector<Unit>& units, int grid_max, int min_pages_per_c
   }
 
 contiguous:
+  grid = ll.grid = grid_cut;
   ll.cta_ptr.clear();
   // Contiguous shares.  Walking the units in order visits the shares in order too, so the items
   // come out already grouped by CTA; share c covers page visits [c W / grid, (c + 1) W / grid),
@@ -1376,7 +1379,16 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
   UnitSlots tile_slots;
   // (fp32: a page of 16 tokens takes a block of 64 rows about 1 us, the merge launch 4 - 5 us)
   if (f32) partition(tile_units, tile_sms * pie_f32_blocks_per_sm(ctx, true), 4, TILE_ROWS, true, plan->tile, &tile_slots, 5);
-  else partition(tile_units, tile_sms, plan->tile_tc ? 32 : 8, TILE_ROWS, true, plan->tile, &tile_slots);
+  else if (!plan->tile_tc) partition(tile_units, tile_sms, 8, TILE_ROWS, true, plan->tile, &tile_slots);
+  else {
+    // tcgen05 row tiles, in units of 16 tokens (about 0.2 us of a CTA; with 8-token pages 0.3): shares of at least 32, a
+    // cut list costs 50 and 0.35 per piece.  Measured, us per step, 32 / 8 heads of 128, 16-token pages, whole against
+    // cut: 64 tokens behind 2,000 35 / 21, 4 x 64 behind 1,000 24 / 33, 4 x 64 behind 3,000 53 / 40, 512 behind 2,000 42 / 48,
+    // 4 x 128 behind 4,000 67 / 58, a prompt of 1,500 32 / 65; whole units on as many CTAs as there are units instead of one
+    // per 512 tokens of the launch: a prompt of 64 tokens 25.6 -> 6.8, one of 300 30.9 -> 10.9 (64-wide heads, 32-token pages).
+    const double k = P == 8 ? 0.7 : 1.0;
+    partition(tile_units, tile_sms, 512 / P, TILE_ROWS, true, plan->tile, &tile_slots, (int)(k * 50 * 16 / P), k * 0.35 * 16 / P);
+  }
   // merge groups of the larger cascaded requests (row-tile items over their private pages): add the slots of
   // the cascade pieces that hold the same rows
   for (PieMerge& m : plan->tile.merges) {
