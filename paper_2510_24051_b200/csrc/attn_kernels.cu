@@ -75,15 +75,21 @@ __device__ __forceinline__ void rows_init(RowState<D>& st, const AttnParams& p, 
   const int row_end = item.row0 + item.nrows;
   st.explicit_mask = rq.mask_row_words != 0;
   st.any_rows = rbase < row_end;
+  const bool one_token = row_end <= p.G;   // (one query token: a row is its place in the head group, no divisions)
   const __nv_bfloat16* qptr[2];
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const int gr = rbase + r_lo + r * 8;
     st.valid[r] = gr < row_end;
-    const int tok = st.valid[r] ? gr / p.G : 0;
-    const int head = item.kv_head * p.G + (st.valid[r] ? gr % p.G : 0);
+    int tok = 0, hg = gr;   // token, place in the head group
+    if (!one_token) {
+      tok = gr / p.G;
+      hg = gr - tok * p.G;
+    }
+    if (!st.valid[r]) tok = hg = 0;
+    const int head = item.kv_head * p.G + hg;
     st.lim[r] = st.valid[r] ? rq.kv_len - rq.q_len + tok : -1;
-    st.hsel[r] = st.valid[r] ? (gr % p.G) / p.G_head : -1;
+    st.hsel[r] = st.valid[r] ? (hg >= p.G_head ? 1 : 0) : -1;   // (a unit covers one or two kv heads)
     st.mrow[r] = p.mask + rq.mask_word_off + (int64_t)tok * rq.mask_row_words;
     qptr[r] = reinterpret_cast<const __nv_bfloat16*>(p.q) + ((int64_t)(rq.q_start + tok) * p.n_q_heads + head) * D;
     st.m_run[r] = kNegInf;
@@ -290,7 +296,12 @@ __device__ __forceinline__ void rows_store(RowState<D>& st, const AttnParams& p,
   for (int r = 0; r < 2; ++r) {
     if (!st.valid[r]) continue;
     const int gr = rbase + r_lo + r * 8;
-    const int tok = gr / p.G, head = item.kv_head * p.G + gr % p.G;
+    int tok = 0, hg = gr;
+    if (item.row0 + item.nrows > p.G) {   // (more than one query token)
+      tok = gr / p.G;
+      hg = gr - tok * p.G;
+    }
+    const int head = item.kv_head * p.G + hg;
     const float L = st.l_run[r];
     const float inv = L > 0.f ? 1.f / L : 0.f;
     const float lse = L > 0.f ? (st.m_run[r] + log2f(L)) * kLn2 : kNegInf;
@@ -925,9 +936,10 @@ __global__ void __launch_bounds__(NW * 32, 1) decode_cluster_kernel(const AttnPa
   // ---- the block's pieces into one partial, then the cluster's partials into the rows
   const int in_block = min(NW, n_pieces - rank * NW), n_blocks = (n_pieces + NW - 1) / NW;
   const int n_vec = item.nrows * (D / 4);   // float4s of the unit's rows
+  const bool one_token = item.row0 + item.nrows <= p.G;
   auto finish = [&](int e, const float4& a, float lse) {   // (every piece of the unit has the same rows)
-    const int row = e / (D / 4), gr = item.row0 + row;
-    const int64_t oi = (int64_t)(item.q_start + gr / p.G) * p.n_q_heads + item.kv_head * p.G + gr % p.G;
+    const int gr = item.row0 + e / (D / 4), tok = one_token ? 0 : gr / p.G;
+    const int64_t oi = (int64_t)(item.q_start + tok) * p.n_q_heads + item.kv_head * p.G + gr - tok * p.G;
     *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + oi * D + (e % (D / 4)) * 4) = make_uint2(pack_bf16(a.x, a.y), pack_bf16(a.z, a.w));
     if (e % (D / 4) == 0) p.lse[oi] = lse;
   };
