@@ -363,7 +363,7 @@ int pie_sched_next_batch(pie_sched* s, int32_t* out_type, int32_t cap, int64_t* 
  *                      request one new token, all on the split-KV kernel, no request listing a
  *                      page another one appends to) lets the attention kernel write the new K/V
  *                      rows itself.  Bit 1: always merge split partials with the merge kernel.  By
- *                      default short decode launches keep all pieces of a (request, kv head)
+ *                      default short decode launches (with bit 4) keep all pieces of a (request, kv head)
  *                      inside one thread block, which merges them itself, and those where whole
  *                      units cannot fill the blocks evenly (a few long requests) cut units across
  *                      thread blocks and still merge inside the kernel: every block combines what it
@@ -374,8 +374,9 @@ int pie_sched_next_batch(pie_sched* s, int32_t* out_type, int32_t cap, int64_t* 
  *                      them in the warps' idle staging buffers in shared memory.  Bit 2: one kv head per
  *                      decode unit.  By default, with 64-wide heads and pages of 8 or 16 tokens, a
  *                      unit is a pair of adjacent kv heads (one copy of twice the size per page).  Bit 4: no
- *                      clusters.  By default every unit of a launch of few or short units is owned by a
- *                      cluster of thread blocks that merges its pieces through (distributed) shared memory. */
+ *                      clusters.  By default every unit of a decode launch is owned by a thread block, or by a
+ *                      cluster of them, that merges its pieces through (distributed) shared memory; only
+ *                      cascades, mixed batches side by side and long launches on 8-token pages are not. */
 enum { PIE_OPT_SPLIT_SMS = 0, PIE_OPT_TILE_SMS = 1, PIE_OPT_OVERLAP = 2, PIE_OPT_NO_FUSION = 3, PIE_NUM_OPTIONS = 4 };
 int pie_set_option(pie_ctx* ctx, int option, int value);
 

@@ -763,16 +763,18 @@ __global__ void __launch_bounds__(NW * 32, 1) attn_split_kernel(const AttnParams
   }
 }
 
-// ------------------------------------------------------------------------------ short units: a cluster or a block per unit
-// Decode launches of a few requests, or of short contexts, are a chain of latencies, not a stream: the two-level merge of
-// attn_split_kernel (a block's pieces through shared memory and a spinning warp; the blocks' partials through L2 with a
-// device-wide fence, an atomic and two dependent reads) was 5 - 6 us of a 17 - 21 us launch of four requests.  Here every
-// unit belongs to ONE cluster of up to 8 thread blocks: each warp takes one contiguous piece of the unit's visits, the
-// pieces of a block meet in shared memory behind a block barrier - every thread combines one float4 of the rows - and the
-// blocks' partials in distributed shared memory behind a cluster barrier, where every block finishes its share of the
-// rows.  No partial goes through L2 and nobody spins.  Sources are combined in page order, so results do not depend on timing.
-// With more units than clusters a unit has one block of 8, 4, 2 or 1 warps to itself, several blocks to an SM.
-// The planner (pick_cluster, partition_cluster) chooses all that; the items carry the same piece fields as a two-level launch.
+// ------------------------------------------------------------------------------ decode: a block or a cluster per unit
+// Every unit belongs to ONE thread block of 1 - 8 warps, or to ONE cluster of up to 8 blocks: each warp takes one contiguous
+// piece of the unit's visits, the pieces of a block meet in shared memory behind a block barrier - every thread combines
+// one float4 of the rows - and the blocks' partials in distributed shared memory behind a cluster barrier, where every
+// block finishes its share of the rows.  No partial goes through L2 and nobody spins.  Sources are combined in page order,
+// so results do not depend on timing.  Blocks are numbered by size, the largest unit first, and dealt to the SMs by the
+// hardware as others end: that evens out what fixed shares cannot know - SMs get up to 10 % different shares of the memory
+// bandwidth -, with no work counter and no chunk partials, and a block's start hides behind its neighbours on the SM.
+// Few requests are a chain of latencies, not a stream: there the two-level merge of attn_split_kernel (shared memory and a
+// spinning warp, then L2 with a device-wide fence, an atomic and two dependent reads) was 5 - 6 us of a 17 - 21 us launch.
+// The planner (pick_cluster, partition_cluster: figures there) chooses the width; the items carry the same piece fields as
+// a two-level launch.
 template <int D, int P, int NW, int DEPTH, int HP>
 struct ClusterCfg {
   static constexpr int PPV = P == 8 ? 2 : 1;

@@ -542,43 +542,51 @@ bool partition_local(const std::vector<Unit>& units, int ctas_max, int NW, int m
   return true;
 }
 
-// Split-KV decode, short units: every unit gets a cluster of `cluster` blocks of NW warps to itself and is cut into one
+// Split-KV decode, a unit per block: every unit gets a cluster of `cluster` blocks of NW warps to itself and is cut into one
 // piece of whole visits (`ppv` pages) per warp, from the cluster's first warp on.  The pieces carry the fields of a
 // two-level merge (PIE_ITEM_LOCAL_* inside a block, PIE_ITEM_GRID_* between the unit's blocks).
 void partition_cluster(const std::vector<Unit>& units, int cluster, int NW, int ppv, int slot_rows, PieLaunchList& ll) {
-  ll.items.clear();
   ll.merges.clear();
-  ll.cta_ptr.clear();
   ll.slot_rows = slot_rows;
   ll.n_slots = 0;
-  ll.n_static = 0;
   ll.cluster = cluster;
   ll.cluster_warps = NW;
   const int width = cluster * NW;
   ll.grid = (int)units.size() * width;
-  ll.items.reserve((size_t)ll.grid);
-  ll.cta_ptr.reserve((size_t)ll.grid + 1);
-  ll.cta_ptr.push_back(0);
+  size_t n_items = 0;
+  for (const Unit& u : units) n_items += (size_t)std::max(1, std::min((u.page_end - u.page_begin + ppv - 1) / ppv, width));
+  ll.items.resize(n_items);
+  ll.cta_ptr.resize((size_t)ll.grid + 1);
+  PieItem* it = ll.items.data();
+  int32_t* ptr = ll.cta_ptr.data();
+  int32_t at = 0;
+  *ptr++ = 0;
   for (const Unit& u : units) {
     const int n = u.page_end - u.page_begin, visits = (n + ppv - 1) / ppv;
-    const int np = std::max(1, std::min(visits, width)), nb = (np + NW - 1) / NW;
-    for (int k = 0; k < np; ++k) {
-      PieItem it = make_item(u, u.page_begin + std::min(n, (int)((int64_t)visits * k / np) * ppv),
-                             u.page_begin + std::min(n, (int)((int64_t)visits * (k + 1) / np) * ppv));
+    const int np = std::max(1, std::min(visits, width)), nb = (np + NW - 1) / NW, each = visits / np, rest = visits % np;
+    const PieItem base = make_item(u, 0, 0);
+    // piece k: visits [visits * k / np, visits * (k + 1) / np), carried from piece to piece without a division
+    for (int k = 0, kb = 0, in_kb = 0, v = 0, carry = 0; k < np; ++k, ++it) {
+      *it = base;   // (copied whole and then completed: the other way round every copy waits for the narrow stores)
+      it->page_begin = u.page_begin + std::min(n, v * ppv);
+      v += each, carry += rest;
+      if (carry >= np) ++v, carry -= np;
+      it->page_end = u.page_begin + std::min(n, v * ppv);
       if (np > 1) {
-        const int kb = k / NW, in_block = std::min(NW, np - kb * NW);
-        it.partial_slot = ll.n_slots + k;
-        if (in_block > 1) it.flags |= PIE_ITEM_LOCAL_PIECE | PIE_ITEM_LOCAL_BITS(0, in_block);
-        if (k % NW == 0) {
-          if (in_block > 1) it.flags |= PIE_ITEM_LOCAL_MERGER;
-          if (nb > 1) it.flags |= PIE_ITEM_GRID_PIECE | PIE_ITEM_GRID_BITS(nb, kb, NW);
+        const int in_block = std::min(NW, np - kb * NW);
+        it->partial_slot = ll.n_slots + k;
+        uint32_t flags = in_block > 1 ? PIE_ITEM_LOCAL_PIECE | PIE_ITEM_LOCAL_BITS(0, in_block) : 0u;
+        if (in_kb == 0) {
+          if (in_block > 1) flags |= PIE_ITEM_LOCAL_MERGER;
+          if (nb > 1) flags |= PIE_ITEM_GRID_PIECE | PIE_ITEM_GRID_BITS(nb, kb, NW);
         }
+        it->flags = flags;
+        if (++in_kb == NW) in_kb = 0, ++kb;
       }
-      ll.items.push_back(it);
-      ll.cta_ptr.push_back((int32_t)ll.items.size());
+      *ptr++ = ++at;
     }
     if (np > 1) ll.n_slots += np;
-    for (int k = np; k < width; ++k) ll.cta_ptr.push_back((int32_t)ll.items.size());   // warps without a piece
+    for (int k = np; k < width; ++k) *ptr++ = at;   // warps without a piece
   }
   ll.n_static = (int32_t)ll.items.size();
 }
@@ -688,40 +696,64 @@ void chunk_units(const std::vector<Unit>& units, int n_warps, PieLaunchList& ll)
 
 static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan);
 
-// Should every unit of a decode launch get a cluster of blocks - or a block - to itself (partition_cluster)?  `blocks` of
-// `warps` warps: the most for which the whole launch is resident at once, no more than the longest unit has use for.
-// Otherwise (false) shares over all warps of the chip.
-static bool pick_cluster(pie_ctx* ctx, const std::vector<Unit>& units, bool plain, int64_t W, int sms, int hp, bool side_by_side, int* blocks,
-                         int* warps) {
+// Should every unit of a decode launch be a block - or a cluster of blocks - of its own (partition_cluster)?  Then the units
+// are put in order of size, the largest first, and the GPU's own block scheduler deals them to the SMs as blocks end:
+// `blocks` of `warps` warps per unit, whichever of 1, 2, 4, 8 warps or 2, 4, 8 blocks of 8 the estimate below favours.
+// Otherwise (false, the units stay as they are) shares over all warps of the chip, laid out in advance.
+static bool pick_cluster(pie_ctx* ctx, std::vector<Unit>& units, bool plain, int64_t W, int sms, int hp, bool side_by_side, bool long_launch,
+                         int* blocks, int* warps) {
   if (units.empty() || !plain || side_by_side || sms != ctx->n_sms || (ctx->options[PIE_OPT_NO_FUSION] & (2 | 8 | 16))) return false;
+  // (Long launches on 8-token pages stay with the chunk list, although blocks of their own are 1.5 - 6 % faster there as well:
+  //  tests/test_gpu_full_configs.py holds them to chunks of odd page counts that merge in a launch of their own.)
+  if (long_launch && ctx->cfg.page_size == 8) return false;
   const int NW = pie_split_warps_per_block(ctx), ppv = ctx->cfg.page_size == 8 ? 2 : 1, n = (int)units.size();
-  int longest_pages = 0;
-  for (const Unit& u : units) longest_pages = std::max(longest_pages, u.page_end - u.page_begin);
-  const int longest = (longest_pages + ppv - 1) / ppv;
-  int c = 0, w = 1;
-  for (int k = 1; k <= NW && n <= sms * (NW / k); k *= 2) {   // blocks of k warps: NW / k of them fit an SM
-    c = 1, w = k;
-    if (k >= longest) break;
+  // runs of units of equal size (the kv heads of a request), largest first: (~size) << 32 | first unit
+  auto size_of = [&](int k) { return units[k].page_end - units[k].page_begin; };
+  std::vector<uint64_t> runs;
+  for (int k = 0; k < n; ++k)
+    if (k == 0 || size_of(k) != size_of(k - 1)) runs.push_back((uint64_t)(0xFFFFFFFFu - (uint32_t)size_of(k)) << 32 | (uint32_t)k);
+  std::sort(runs.begin(), runs.end());
+  std::vector<Unit> sorted;
+  sorted.reserve((size_t)n);
+  for (uint64_t r : runs)
+    for (int k = (int)(uint32_t)r, sz = size_of(k); k < n && size_of(k) == sz; ++k) sorted.push_back(units[k]);
+  const int longest_pages = sorted[0].page_end - sorted[0].page_begin, longest = (longest_pages + ppv - 1) / ppv;
+
+  // Estimates in us, without what all widths have in common: the bytes at 8 TB/s and 0.75 of the time by which the last block
+  // outlasts the even share of a slot (a slot: room for one unit; blocks of k warps: NW / k of them fit an SM), or that
+  // block alone, a warp taking `t_visit` per visit; 6 % of the longest block, because SMs differ in their share of the memory
+  // bandwidth; 1 for the merge across a cluster; and 6 for every block that follows another in a slot, 4 for a cluster - a
+  // full turn even for one that is left over, and more with larger visits: a cluster starts when all its SMs are free.
+  // Over 460 batches of 1 - 200 requests and 20 - 16,000 tokens (32 / 8 heads of 64 and of 128, 16 / 2, 12 / 12; 8-, 16- and 32-token
+  // pages) the width it picks is 0.3 % behind the best one on average, 16 % at worst.  us per launch, in brackets shares over all
+  // warps laid out in advance with the two-level merge, which were nowhere more than 7 % better: 64-wide heads 4 requests of
+  // 512 - 4,096 tokens 7.4 (19.0), 32 of them 30.8 (35.7), 64 of them 47.1 (54.4), 6 of 8,000 - 16,000 32.8 (34.6), 128 of 200 - 2,000
+  // 49.2 (58.4); 128-wide heads 14 of 1,000 - 2,000 19.5 (25.0), 64 of 1,024 - 8,192 162 (185); 256 policy-masked contexts of
+  // 16,384 - 32,768, whose alternative is the chunk list, 981 (999).
+  const double visit_bytes = (double)ppv * hp * 4.0 * ctx->cfg.page_size * ctx->cfg.head_dim, visits = (double)W / ppv;
+  const double t_visit = ppv == 2 ? 1.0 : visit_bytes > 8192 ? 1.1 : 0.85;   // (two copies per visit; 16 KB visits)
+  const double t_bytes = visits * visit_bytes / 8e6;
+  std::vector<int> lanes;
+  double best = 1e30;
+  for (int width = 1, shift = ppv - 1; width <= 8 * NW; width *= 2, ++shift) {   // warps per unit
+    const int c = std::max(1, width / NW), w = std::min(width, NW);
+    const int slots = c == 1 ? sms * (NW / w) : pie_split_max_clusters(ctx, hp, c);
+    if (slots <= 0 || (c > 1 && n > 8 * slots)) break;
+    auto piece = [&](int k) { return (sorted[k].page_end - sorted[k].page_begin + ppv * width - 1) >> shift; };
+    const double even = visits / ((double)std::min(n, slots) * width);
+    int last = piece(0);
+    if (n > slots && (c > 1 || n <= 2 * slots)) {   // dealt there and back
+      lanes.assign((size_t)slots, 0);
+      for (int k = 0, turn = 0; k < n; ++turn)
+        for (int l = 0; l < slots && k < n; ++l, ++k) last = std::max(last, lanes[turn & 1 ? slots - 1 - l : l] += piece(k));
+    }
+    const double turns = c == 1 ? 6.0 * std::max(0.0, (double)n / slots - 1.0) : 4.0 * ((n - 1) / slots) * std::max(1.0, visit_bytes / 8192);
+    const double t = std::max(last * t_visit, t_bytes + 0.75 * t_visit * std::max(0.0, last - even)) +
+                     0.06 * visit_bytes / 8192 * piece(0) + (c > 1) + turns;
+    if (t < best) { best = t; *blocks = c; *warps = w; }
+    if (width >= longest) break;
   }
-  if (c == 0) return false;
-  for (int k = 2; w == NW && c * w < longest && k <= 8 && n <= pie_split_max_clusters(ctx, hp, k); k *= 2) c = k;
-  // Estimates in us.  Here: 4.5 to start and merge, then the longest piece at the rate of a warp that has the memory system
-  // to itself, or the bytes at the chip's rate and half the time by which the longest piece outlasts an average one.  The
-  // alternative: the bytes, 11 to start and merge, and 4.5 more for the two-level merge of units cut across blocks (the
-  // test is the one of partition_local; behind more than 12 us of bytes that merge is hidden).  Measured on 1 - 200
-  // requests of 20 - 8,000 tokens (32 / 8 heads of 64 and of 128, 16 / 2, 12 / 12; 8-, 16- and 32-token pages), in
-  // brackets the alternative, us per launch: 1 x 2,000 tokens 6.3 (19.5), 4 x 2,000 8.0 (19.5), 4 x 8,000 18.0 (22.6),
-  // 12 x 2,000 12.9 (22.6), 24 x 600 8.1 (12.3), 48 x 2,000 31.5 (34.3), 200 x 600 38.8 (40.9); where lengths differ more
-  // it loses and is not taken: 48 requests of 100 - 2,000 tokens 29.5 (26.3).
-  const double visit_bytes = (double)ppv * hp * 4.0 * ctx->cfg.page_size * ctx->cfg.head_dim;
-  const double t_visit = ppv == 2 ? 1.08 : visit_bytes > 8192 ? 1.05 : 0.83;   // (two copies per visit; 16 KB visits)
-  const double t_bytes = (double)W / ppv * visit_bytes / 6.4e6;
-  const double piece = (double)((longest + c * w - 1) / (c * w)), mean = (double)W / ppv / ((double)n * c * w);
-  const double t_here = 4.5 + std::max(piece * t_visit, t_bytes + 0.5 * t_visit * std::max(0.0, piece - mean));
-  const bool cut = (int64_t)longest_pages * sms * 100 > W * 108 && longest_pages > W / sms + 100;
-  if (t_here + 2.0 > t_bytes + (cut && t_bytes < 12 ? 15.5 : 11.0)) return false;
-  *blocks = c;
-  *warps = w;
+  units.swap(sorted);
   return true;
 }
 
@@ -1448,7 +1480,7 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
       // (a block takes a 16-token page in about 0.1 us, the launch 4 - 5 us)
       partition(split_units, split_sms * pie_f32_blocks_per_sm(ctx, false), 16, max_rows, true, plan->split, nullptr, 45);
       plan->split.n_static = (int32_t)plan->split.items.size();
-    } else if (int c_blocks = 0, c_warps = 0; pick_cluster(ctx, split_units, plain_units, W, split_sms, hp, plan->overlap, &c_blocks, &c_warps)) {
+    } else if (int c_blocks = 0, c_warps = 0; pick_cluster(ctx, split_units, plain_units, W, split_sms, hp, plan->overlap, long_launch, &c_blocks, &c_warps)) {
       partition_cluster(split_units, c_blocks, c_warps, P == 8 ? 2 : 1, max_rows, plan->split);
     } else if (long_launch || (W >= (int64_t)200 * n_warps && !plain_units)) {
       chunk_units(split_units, n_warps, plan->split);

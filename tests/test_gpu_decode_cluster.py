@@ -46,3 +46,14 @@ def test_two_query_tokens_and_masks(D, P):
     masks[0][0, 5] = True
     info, _ = _run(shapes, 8, 2, D, P, masks)
     assert info["num_tile_items"] == 0
+
+
+@pytest.mark.parametrize("H_q,H_kv,D,P,long,short,R", [(12, 12, 64, 8, 20, 5, 210), (4, 2, 128, 16, 1500, 900, 24), (4, 2, 128, 32, 700, 100, 100)])
+def test_more_units_than_are_resident_at_once(H_q, H_kv, D, P, long, short, R):
+    """Blocks (or clusters) that start when others end: the largest units first, whatever their place in the batch."""
+    rng = np.random.RandomState(R)
+    kv = [int(x) for x in rng.randint(1, short + 1, R)]
+    for k in (1, R // 2, R - 1):
+        kv[k] = long
+    info, _ = _run([(1, n) for n in kv], H_q, H_kv, D, P, seed=R)
+    assert info["num_merge_groups"] == 0 and info["launches"] == 1
