@@ -3,24 +3,29 @@
 //
 // One CTA per SM walks its share of work items.  An item is up to 256 rows (row = query token *
 // G + head-in-group, one kv head) = two 128-row Q tiles, attended over the item's kept pages in
-// KV tiles of 128 tokens that are handled as two halves of 64 columns.  Roles (352 threads):
-//   warps 0-3 / 4-7  softmax warpgroup of Q tile 0 / 1: one row per thread.  Reads a half of S
-//                    from TMEM, masks, exponentiates, writes bf16 P back over that half of S,
-//                    keeps the running (max, sum), rescales O in TMEM only when the row max grew
-//                    by more than 2^8, and runs the epilogue.
-//   warp 8           producer: linear bulk copies of page blocks into the K / V stage rings.  The
+// KV tiles of 128 tokens that are handled as two halves of 64 columns.  Roles (a warp each behind the softmax warpgroups):
+//   warpgroups       softmax of Q tile 0 / 1: one row per thread.  Reads a half of S from TMEM, masks, exponentiates, writes
+//                    bf16 P back over that half of S, keeps the running (max, sum), rescales O in TMEM only when the row max
+//                    grew by more than 2^8, and runs the epilogue.  128-wide heads: two warpgroups, one per Q tile, that
+//                    take both halves in turn.  64-wide heads: FOUR, one per (Q tile, half), each with an accumulator of
+//                    its own, that meet in the epilogue.  There the exponentials bound the kernel (2,048 cycles per KV tile
+//                    of the two Q tiles at 16 per cycle and SM, the MMAs half of that), and two warps per scheduler left
+//                    that pipe idle in the waits of each half: 2,900 cycles per KV tile; four take 2,500.  us per launch,
+//                    32 / 8 heads, before -> now: 8 chunks of 512 behind 4,096 135 -> 122, 40 behind 2,048 368 -> 337, two
+//                    prompts of 4,000 201 -> 185, 37 chunks of 64 behind 8,000 117 -> 106.  (128-wide heads fill TMEM with two.)
+//   producer         linear bulk copies of page blocks into the K / V stage rings.  The
 //                    pool's storage order is the 128-byte-swizzled canonical operand layout, so a
 //                    page block drops into its 16-row band of the tile with no tensor map.
-//   warp 9, one lane MMA issuer: S_t^h = Q_t K_h^T (N = 64), O_t += P_t^h V_h with tcgen05.mma,
+//   issuer, one lane MMAs: S_t^h = Q_t K_h^T (N = 64), O_t += P_t^h V_h with tcgen05.mma,
 //                    accumulators and P in TMEM; completion is tracked with tcgen05.commit.
-//   warp 10          Q loader (TMA): runs one item ahead, so that the first S of the next item is
+//   Q loader (TMA)   runs one item ahead, so that the first S of the next item is
 //                    computed while the warpgroups are still in the epilogue of this one.
 // The tensor pipe takes instructions synchronously from the issuing thread (measured: a group of
 // eight MMAs returns after ~8 x 64 cycles and any other work of that thread is idle pipe time), so
 // the issuer is a single thread that does nothing but wait, issue and commit.  The two halves
 // break the chain S -> softmax -> PV -> next S of a Q tile: while a warpgroup works on one half,
 // the PV of the other half and the next S into the columns it frees are already running.
-// TMEM (512 columns): S0a S0b | S1a S1b | O0 | O1; P_t^h overlays the first 32 columns of S_t^h.
+// TMEM (512 columns): S0a S0b | S1a S1b | O0 | O1 (64-wide heads: O0a O0b O1a O1b); P_t^h overlays the first 32 columns of S_t^h.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -88,9 +93,9 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 // every bulk store of this thread has finished READING shared memory / has completed altogether
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-// barrier among the 128 threads of one softmax warpgroup (ids 1 and 2; 0 is __syncthreads)
-template <int ID>
-__device__ __forceinline__ void wg_sync() { asm volatile("bar.sync %0, 128;" ::"n"(ID) : "memory"); }
+// barrier among the N softmax threads of one Q tile (ids 1 and 2; 0 is __syncthreads)
+template <int ID, int N>
+__device__ __forceinline__ void wg_sync() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
@@ -170,7 +175,6 @@ constexpr float kLn2 = 0.6931471805599453f;
 constexpr int kTileM = 128;    // rows per Q tile
 constexpr int kTileN = 128;    // tokens per KV tile (one stage of the K / V rings)
 constexpr int kHalf = 64;      // columns per half tile: the unit handed between softmax and MMA
-constexpr int kThreads = 352;
 
 template <int D, int P>
 struct TcCfg {
@@ -183,13 +187,18 @@ struct TcCfg {
   static constexpr int QTILE = kTileM * D * 2;
   static constexpr int KVTILE = kTileN * D * 2;
   static constexpr int STAGES = D == 128 ? 2 : 4;
+  // 64-wide heads: FOUR softmax warpgroups, one per (Q tile, half), each with an accumulator of its own (4 x 64 columns of S,
+  // 4 x 64 of O: all of TMEM); the two partial results of a row meet in the epilogue.
+  static constexpr bool SPLIT = D == 64;
+  static constexpr int NWG = SPLIT ? 4 : 2;            // softmax warpgroups; the roles behind them have one warp each
+  static constexpr int THREADS = NWG * 128 + 96;
   static constexpr int NBAR = 4 * STAGES + 19;
   static constexpr int OSLAB = kTileM * 128;           // output staging: one 64-column slab of a 128-row tile per warpgroup
-  static constexpr int SMEM = 2 * QTILE + 2 * STAGES * KVTILE + 2 * OSLAB + NBAR * 8 + 64;
+  static constexpr int SMEM = 2 * QTILE + 2 * STAGES * KVTILE + 2 * OSLAB + NBAR * 8 + 64 + (SPLIT ? 8 * kTileM * 8 : 0);
 };
 
 template <int D, int P>
-__global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p, const __grid_constant__ CUtensorMap qmap,
+__global__ void __launch_bounds__(TcCfg<D, P>::THREADS, 1) attn_tc_kernel(const AttnParams p, const __grid_constant__ CUtensorMap qmap,
                                                               const __grid_constant__ CUtensorMap omap, const int kflags) {
   using C = TcCfg<D, P>;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -208,9 +217,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
   uint64_t* p_full = s_full + 4;           // [2][2]   P_t^h is written (128 arrivals)
   uint64_t* pv_done = p_full + 4;          // [2]      one phase per PV group of Q tile t
   uint64_t* o_done = pv_done + 2;          // [2]      last PV of the item is complete
-  uint64_t* o_free = o_done + 2;           // [2]      the epilogue has read O_t (128 arrivals)
+  uint64_t* o_free = o_done + 2;           // [2]      the epilogue has read O_t (128 arrivals a warpgroup)
   uint64_t* v_land = o_free + 2;           // [1]      producer-private: V tile that needs its tail cleared
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(v_land + 1);
+  float2* sML = reinterpret_cast<float2*>(tmem_slot + 2);   // SPLIT: [2 buffers][2 Q tiles][2 halves][128 rows] (reference, sum)
+  constexpr int kProducer = 4 * C::NWG, kIssuer = kProducer + 1, kLoader = kProducer + 2;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool use_qmap = kflags & 1;      // Q tiles come through the tensor map
@@ -232,12 +243,12 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
       }
       mbar_init(smem_u32(pv_done + t), 1);
       mbar_init(smem_u32(o_done + t), 1);
-      mbar_init(smem_u32(o_free + t), kTileM);
+      mbar_init(smem_u32(o_free + t), C::SPLIT ? 2 * kTileM : kTileM);
     }
     mbar_init(smem_u32(v_land), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 8) {
+  if (warp == kProducer) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -250,7 +261,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
 
   const int it0 = p.cta_ptr[blockIdx.x], it1 = p.cta_ptr[blockIdx.x + 1];
 
-  if (warp == 8) {
+  if (warp == kProducer) {
     // ================================================================ producer
     uint32_t tile_cnt = 0, land_cnt = 0;
     for (int it = it0; it < it1; ++it) {
@@ -308,7 +319,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
         }
       }
     }
-  } else if (warp == 9) {
+  } else if (warp == kIssuer) {
     // ================================================================ MMA issuer
     // One elected lane runs the whole role.  (Electing the lane, rather than testing the lane id,
     // lets the compiler keep descriptors and loop state in uniform registers; measured, it halves
@@ -397,11 +408,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
               for (int t = 0; t < 2; ++t) {
                 mbar_wait(bar_p + 8 * (2 * t + h), (half_ph >> (2 * t + h)) & 1, p.status);
                 tc_fence_after();
-                const uint32_t dO = tmem + 256 + t * D, dS = tmem + t * 128 + h * kHalf;
+                const uint32_t dO = tmem + 256 + (C::SPLIT ? 2 * t + h : t) * D, dS = tmem + t * 128 + h * kHalf;
 #pragma unroll
                 for (int ks = 0; ks < kHalf / 16; ++ks)   // 16 token rows = 2048 bytes per k-step
                   umma_ts(dO, dS + ks * 8, vd0 + (uint64_t)((h * (kHalf / 16) + ks) * 128), idesc_pv, 1u);
-                umma_commit(bar_pv + 8 * t);
+                if (!C::SPLIT) umma_commit(bar_pv + 8 * t);
                 if (h == 1 && t == 1) umma_commit(smem_u32(v_empty + s));
                 const uint64_t qd = q_desc0 + (uint64_t)(t * (C::QTILE >> 4));
                 const uint64_t kd = kd0 + (uint64_t)(h * ((kHalf * 128) >> 4));
@@ -431,13 +442,13 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
                 mbar_wait(smem_u32(k_full + sn), phn, p.status);
                 k_ready = true;
               }
-              if (i == 0) mbar_wait(smem_u32(o_free + t), ((ph_item >> t) & 1) ^ 1, p.status);  // the previous epilogue has drained O_t
+              if (C::SPLIT ? j == 0 : i == 0) mbar_wait(smem_u32(o_free + t), ((ph_item >> t) & 1) ^ 1, p.status);  // the previous epilogue has drained O_t
               tc_fence_after();
               const uint64_t vd = v_desc0 + (uint64_t)(s * (C::KVTILE >> 4) + h * (kHalf / 16) * 128);
-              const uint32_t dO = tmem + 256 + t * D, aP = tmem + t * 128 + h * kHalf;
+              const uint32_t dO = tmem + 256 + (C::SPLIT ? 2 * t + h : t) * D, aP = tmem + t * 128 + h * kHalf;
               for (int ks = 0; ks < ksteps; ++ks)
-                umma_ts(dO, aP + ks * 8, vd + (uint64_t)(ks * 128), idesc_pv, (i > 0 || ks > 0) ? 1u : 0u);
-              umma_commit(bar_pv + 8 * t);
+                umma_ts(dO, aP + ks * 8, vd + (uint64_t)(ks * 128), idesc_pv, ((C::SPLIT ? j > 0 : i > 0) || ks > 0) ? 1u : 0u);
+              if (!C::SPLIT) umma_commit(bar_pv + 8 * t);
               if (h == nh - 1 && t == nt - 1) umma_commit(smem_u32(v_empty + s));
               if (i + 1 == nhalf) umma_commit(smem_u32(o_done + t));
               if (h < nhn) {   // S_t^h of the next tile goes into the columns this PV frees
@@ -452,8 +463,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
         tile_cnt += ntiles;
       }
     }
-  } else if (warp >= 10) {
-    // ================================================================ Q loader (warp 10)
+  } else if (warp == kLoader) {
+    // ================================================================ Q loader
     // Runs one item ahead: the next item's Q rows go into shared memory (K-major, 128-byte
     // swizzle) as soon as the S MMAs of the current item no longer read the tile.  A Q tile is
     // the box (64 dims, G heads of the group, 128 / G tokens) of the Q tensor: two TMA loads per
@@ -503,34 +514,42 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
     }
   } else {
     // ================================================================ softmax warpgroups
-    const int t = warp >> 2;                       // Q tile of this warpgroup
+    const int t = (warp >> 2) & 1;                 // Q tile of this warpgroup
+    const int hw = warp >> 3;                      // SPLIT: the half of every KV tile it takes (otherwise 0: both)
     const int rho = (warp & 3) * 32 + lane;        // row inside the tile = TMEM lane
     const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;
-    const uint32_t tS = tmem + t * 128 + lane_sel, tO = tmem + 256 + t * D + lane_sel;
+    const uint32_t tS = tmem + t * 128 + lane_sel, tO = tmem + 256 + (C::SPLIT ? 2 * t + hw : t) * D + lane_sel;
     uint32_t my_items = 0;   // phase of o_done
     uint32_t s_ph = 0;       // bit h: phase of s_full[t][h]
     uint32_t n_arr = 0;      // p_full arrivals so far = PV groups of this Q tile issued or about to be
-    // The record of the next item is fetched before the wait for the last PV of the current one, so that its
-    // latency is not added to the gap between two items (where the tensor pipe is idle).
-    PieItem item_nxt = PieItem{};
-    if (it0 < it1) item_nxt = p.items[it0];
+    // An item's record is held by the warp as one word per lane, and a field is a shuffle: one register instead of 16, so that
+    // the next record can be fetched before the wait for the last PV of the current one - its latency is not added to the gap
+    // between two items, in which the exponentials and the tensor pipe stand still.
+    auto fetch_item = [&](int k) { return k < it1 && lane < 16 ? ldg_early(reinterpret_cast<const uint32_t*>(p.items + k) + lane) : 0u; };
+    uint32_t words_nxt = fetch_item(it0);
     for (int it = it0; it < it1; ++it) {
-      const PieItem item = item_nxt;
-      const int npages = item.page_end - item.page_begin;
+      const uint32_t words = words_nxt;
+      auto field = [&](size_t offset) { return (int)__shfl_sync(0xFFFFFFFFu, words, (int)(offset / 4)); };
+#define ITEM(f) field(offsetof(PieItem, f))
+      const int page_begin = ITEM(page_begin), npages = ITEM(page_end) - page_begin, nrows = ITEM(nrows);
       const int nhalf = (npages + C::PPH - 1) / C::PPH;
-      const int nt = item.nrows > kTileM ? 2 : 1;
+      const int n_own = C::SPLIT ? (nhalf - hw + 1) / 2 : nhalf;   // halves of this warpgroup: own half n is half_of(n) of the item
+      auto half_of = [&](int n) { return C::SPLIT ? 2 * n + hw : n; };
+      const int nt = nrows > kTileM ? 2 : 1;
       if (t >= nt) {
-        if (it + 1 < it1) item_nxt = p.items[it + 1];
+        words_nxt = fetch_item(it + 1);
         continue;
       }
-      const int gr = item.row0 + t * kTileM + rho;
-      const bool valid = gr < item.row0 + item.nrows;
-      const int tok = valid ? gr / p.G : 0;
-      const int head = item.kv_head * p.G + (valid ? gr % p.G : 0);
-      const int64_t oi = (int64_t)(item.q_start + tok) * p.n_q_heads + head;
-      const int lim = valid ? item.kv_len - item.q_len + tok : -1;
-      const uint32_t* mrow = p.mask + item.mask_word_off + (int64_t)tok * item.mask_row_words;
-      const bool explicit_mask = item.mask_row_words != 0;
+      // (rows past the end of the item are computed like a row of its first token - what Q holds there is some other
+      //  row or zero - and not stored: left without any column they would keep their warp off the lean path)
+      const int gr = t * kTileM + rho;
+      const int row0 = ITEM(row0), mask_row_words = ITEM(mask_row_words);
+      const int tok = gr < nrows ? (row0 + gr) / p.G : row0 / p.G;
+      const int lim = ITEM(kv_len) - ITEM(q_len) + tok;
+      const int64_t mask_word_off = (int64_t)((uint64_t)(uint32_t)field(offsetof(PieItem, mask_word_off)) |
+                                              (uint64_t)(uint32_t)field(offsetof(PieItem, mask_word_off) + 4) << 32);
+      const uint32_t* mrow = p.mask + mask_word_off + (int64_t)tok * mask_row_words;
+      const bool explicit_mask = mask_row_words != 0;
       float m_ref = kNegInf, l_sum = 0.f;
 
       if (nhalf > 0) {
@@ -538,7 +557,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
         // allowed-position bits of this row run two halves ahead of the softmax.  The loads are
         // volatile so that they are issued here and not next to their first use, where their
         // latency would be exposed on every half.
-        const int2* krec = p.kept + item.page_begin;
+        const int2* krec = p.kept + page_begin;
         auto load_recs = [&](int i, uint32_t* rec) {
 #pragma unroll
           for (int g = 0; g < C::PPH; ++g) {
@@ -547,38 +566,41 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
             if (pg < npages) rec[g] = ldg_early(reinterpret_cast<const uint32_t*>(&krec[pg].y));
           }
         };
+        // (one bit per column, a word per 32-column chunk)
         auto make_bits = [&](const uint32_t* rec, uint32_t* bits) -> bool {
-          uint32_t any = valid ? 0u : PIE_KEPT_NEEDS_MASK;
+          uint32_t any = 0u;
 #pragma unroll
           for (int g = 0; g < C::PPH; ++g) any |= rec[g];
-          if (!(any & PIE_KEPT_NEEDS_MASK)) return false;   // common case: every page fully visible (warp-uniform unless rows are padding)
+          if (!(any & PIE_KEPT_NEEDS_MASK)) return false;   // common case: every page fully visible (warp-uniform)
+          constexpr uint32_t kPage = P == 32 ? 0xFFFFFFFFu : (1u << (P & 31)) - 1u;
+          bits[0] = bits[1] = 0u;
 #pragma unroll
           for (int g = 0; g < C::PPH; ++g) {
             const uint32_t lpf = rec[g];
-            bits[g] = 0xFFFFFFFFu;
-            if (lpf == 0xFFFFFFFFu || !valid) {
-              bits[g] = 0u;
+            uint32_t b = kPage;
+            if (lpf == 0xFFFFFFFFu) {
+              b = 0u;
             } else if (lpf & PIE_KEPT_NEEDS_MASK) {
               const int j0 = (int)(lpf & ~PIE_KEPT_NEEDS_MASK) * P;
-              if (explicit_mask) bits[g] = ldg_early(mrow + (j0 >> 5)) >> (j0 & 31);
-              else bits[g] = lim >= j0 + P - 1 ? 0xFFFFFFFFu : (lim < j0 ? 0u : ((1u << (lim - j0 + 1)) - 1u));
+              if (explicit_mask) b = (ldg_early(mrow + (j0 >> 5)) >> (j0 & 31)) & kPage;
+              else b = lim >= j0 + P - 1 ? kPage : (lim < j0 ? 0u : ((1u << (lim - j0 + 1)) - 1u));
             }
+            bits[g * P / 32] |= b << (g * P % 32);
           }
           return true;
         };
         // Halves that lie inside the item's clean prefix (pages every row of the tile sees in full,
         // counted by the planner) need neither records nor bits; the look-ahead starts two halves
         // before the first half that does.
-        const int clean_halves = (int)(item.flags >> PIE_ITEM_CLEAN_SHIFT) / C::PPH;
-        uint32_t rec_nxt[C::PPH], bits_nxt[C::PPH], bits[C::PPH];
-#pragma unroll
-        for (int g = 0; g < C::PPH; ++g) bits_nxt[g] = 0xFFFFFFFFu;
+        const int clean_item = (int)((uint32_t)ITEM(flags) >> PIE_ITEM_CLEAN_SHIFT) / C::PPH;
+        const int clean_halves = C::SPLIT ? (clean_item - hw + 1) / 2 : clean_item;   // (of this warpgroup)
+        uint32_t rec_nxt[C::PPH], bits_nxt[2] = {0xFFFFFFFFu, 0xFFFFFFFFu}, bits[2];
         bool mask_nxt = false;
         if (clean_halves <= 0) {
-          load_recs(0, rec_nxt);
+          load_recs(half_of(0), rec_nxt);
           mask_nxt = make_bits(rec_nxt, bits_nxt);
         }
-        if (clean_halves <= 1) load_recs(1, rec_nxt);
+        if (clean_halves <= 1) load_recs(half_of(1), rec_nxt);
 
         // P = exp2(x * scale - m) for one chunk of 32 columns: bf16 pairs into pk, the sums onto sa / sb.
         auto exp_chunk = [&](const float* x, const uint64_t scale2, const uint64_t negm2, uint64_t& sa, uint64_t& sb, uint32_t* pk) {
@@ -596,18 +618,18 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
         };
         // One half of the item.  The body exists twice: a lean copy for the halves of the clean
         // prefix (no records, no bits, no masking code in the loop) and the general one.
-        auto do_half = [&](const int i, auto masked_tag) {
+        auto do_half = [&](const int i, auto masked_tag) {   // i: own half
           constexpr bool kMasked = decltype(masked_tag)::value;
-          const int h = i & 1;
+          const int h = C::SPLIT ? hw : i & 1;
           const uint32_t tSh = tS + h * kHalf;
           bool half_mask = false;
           if constexpr (kMasked) {
             half_mask = mask_nxt;
-#pragma unroll
-            for (int g = 0; g < C::PPH; ++g) bits[g] = bits_nxt[g];
+            bits[0] = bits_nxt[0];
+            bits[1] = bits_nxt[1];
             mask_nxt = false;
             if (i + 1 >= clean_halves) mask_nxt = make_bits(rec_nxt, bits_nxt);   // half i + 1 (all "no such page" past the end)
-            if (i + 2 >= clean_halves) load_recs(i + 2, rec_nxt);
+            if (i + 2 >= clean_halves) load_recs(half_of(i + 2), rec_nxt);
           }
 
           mbar_wait(smem_u32(s_full + 2 * t + h), (s_ph >> h) & 1, p.status);
@@ -618,19 +640,21 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
           // lag the true running maximum by up to 2^8; when a chunk exceeds that (rare after the first
           // chunk of an item), O_t, the sums and the P chunk already written for this half are brought
           // to the new reference.  Scale-and-shift and the row sum use packed fp32x2 arithmetic.
-          uint64_t psum_a = pack_f32x2(0.f, 0.f), psum_b = pack_f32x2(0.f, 0.f);
           const uint64_t scale2 = pack_f32x2(p.scale_log2, p.scale_log2);
-          float xbuf[2][32];   // double buffer: chunk 1 is in flight while chunk 0 is processed
+          // two buffers: chunk 1 is in flight while chunk 0 is processed (four warps per scheduler cover that latency, and
+          // have 104 registers a thread: one buffer)
+          constexpr int kBuf = C::SPLIT ? 1 : 2;
+          float xbuf[kBuf][32];
           tmem_ld32(tSh, reinterpret_cast<uint32_t*>(xbuf[0]));
           tmem_wait_ld();
 #pragma unroll
           for (int k = 0; k < kHalf / 32; ++k) {
-            float* x = xbuf[k & 1];
-            if (k + 1 < kHalf / 32) tmem_ld32(tSh + (k + 1) * 32, reinterpret_cast<uint32_t*>(xbuf[(k + 1) & 1]));
+            float* x = xbuf[k % kBuf];
+            if (kBuf == 2 && k + 1 < kHalf / 32) tmem_ld32(tSh + (k + 1) * 32, reinterpret_cast<uint32_t*>(xbuf[(k + 1) % kBuf]));
             if (kMasked && half_mask) {
 #pragma unroll
               for (int c = 0; c < 32; ++c)
-                if (!((bits[(k * 32 + c) / P] >> ((k * 32 + c) % P)) & 1u)) x[c] = kNegInf;
+                if (!((bits[k] >> c) & 1u)) x[c] = kNegInf;
             }
             // Lean form (the whole of the lean copy; in the general copy the first attempt on every chunk, masked
             // scores being -inf by now - the halves around an item's first masked page and the diagonal of a
@@ -639,7 +663,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
             // sum below 2^16 proves that no score runs ahead of the reference by more than 16 binades
             // (fp32 sums and bf16 P keep their relative precision at any such lag).  Otherwise - or when a
             // row of the warp has no reference yet - the chunk is redone the careful way below.
-            if constexpr (!kMasked || P != 8) {   // (with 8-token pages the general loop has no registers left for it)
+            {
               if (__all_sync(0xFFFFFFFFu, m_ref != kNegInf)) {
                 const uint64_t negm2 = pack_f32x2(-m_ref, -m_ref);
                 uint64_t ca = pack_f32x2(0.f, 0.f), cb = pack_f32x2(0.f, 0.f);
@@ -648,9 +672,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
                 float s0, s1;
                 unpack_f32x2(add_f32x2(ca, cb), s0, s1);
                 if (!__any_sync(0xFFFFFFFFu, !(s0 + s1 <= 65536.f))) {   // (also catches inf and NaN)
-                  psum_a = add_f32x2(psum_a, ca);
-                  psum_b = add_f32x2(psum_b, cb);
+                  l_sum += s0 + s1;
                   tmem_st16(tSh + k * 16, pk);
+                  if (kBuf == 1 && k + 1 < kHalf / 32) tmem_ld32(tSh + (k + 1) * 32, reinterpret_cast<uint32_t*>(xbuf[0]));
                   if (k + 1 < kHalf / 32) tmem_wait_ld();
                   continue;
                 }
@@ -668,14 +692,15 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
               const float f = (m_ref == kNegInf) ? 1.f : fast_exp2(m_ref - m_new);
               if (m_new != kNegInf) m_ref = m_new;
               l_sum *= f;
-              psum_a = fma_f32x2(psum_a, pack_f32x2(f, f), pack_f32x2(0.f, 0.f));
-              psum_b = fma_f32x2(psum_b, pack_f32x2(f, f), pack_f32x2(0.f, 0.f));
               if (i > 0) {
                 // O_t holds the PV groups of halves 0..i-1; the latest may still be running.  All but
                 // the latest are known complete (S_t^h of this half was issued after them), so the
                 // barrier is at most one phase behind and the parity wait is unambiguous.
-                mbar_wait(smem_u32(pv_done + t), (n_arr - 1) & 1, p.status);
-                tc_fence_after();
+                // (SPLIT: S of this half was issued after the latest PV of this accumulator, so that one is complete.)
+                if (!C::SPLIT) {
+                  mbar_wait(smem_u32(pv_done + t), (n_arr - 1) & 1, p.status);
+                  tc_fence_after();
+                }
 #pragma unroll 1
                 for (int c0 = 0; c0 < D; c0 += 16) {
                   uint32_t o[16];
@@ -703,129 +728,176 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
             }
             const float neg_m = (m_ref == kNegInf) ? 0.f : -m_ref;
             const uint64_t negm2 = pack_f32x2(neg_m, neg_m);
+            uint64_t ca = pack_f32x2(0.f, 0.f), cb = pack_f32x2(0.f, 0.f);
             uint32_t pk[16];
-            exp_chunk(x, scale2, negm2, psum_a, psum_b, pk);
-            tmem_st16(tSh + k * 16, pk);   // columns [16k, 16k+16): below every S column still to be read
-            if (k + 1 < kHalf / 32) tmem_wait_ld();
-          }
-          {
+            exp_chunk(x, scale2, negm2, ca, cb, pk);
             float s0, s1;
-            unpack_f32x2(add_f32x2(psum_a, psum_b), s0, s1);
+            unpack_f32x2(add_f32x2(ca, cb), s0, s1);
             l_sum += s0 + s1;
+            tmem_st16(tSh + k * 16, pk);   // columns [16k, 16k+16): below every S column still to be read
+            if (kBuf == 1 && k + 1 < kHalf / 32) tmem_ld32(tSh + (k + 1) * 32, reinterpret_cast<uint32_t*>(xbuf[0]));
+            if (k + 1 < kHalf / 32) tmem_wait_ld();
           }
           tmem_wait_st();
           tc_fence_before();
           mbar_arrive(smem_u32(p_full + 2 * t + h));
           ++n_arr;
         };
-        const int n_lean = min(nhalf, max(0, clean_halves - 2));   // (the look-ahead of the general loop starts two halves early)
+        const int n_lean = min(n_own, max(0, clean_halves - 2));   // (the look-ahead of the general loop starts two halves early)
         for (int i = 0; i < n_lean; ++i) do_half(i, std::false_type{});
-        for (int i = n_lean; i < nhalf; ++i) do_half(i, std::true_type{});
-        if (it + 1 < it1) item_nxt = p.items[it + 1];
-        mbar_wait(smem_u32(o_done + t), my_items & 1, p.status);
-        ++my_items;
-        tc_fence_after();
+        for (int i = n_lean; i < n_own; ++i) do_half(i, std::true_type{});
       }
-
-      if (nhalf == 0 && it + 1 < it1) item_nxt = p.items[it + 1];
+      words_nxt = fetch_item(it + 1);
+      const int kv_head = ITEM(kv_head), q_start = ITEM(q_start), partial_slot = ITEM(partial_slot), e_row0 = ITEM(row0), e_nrows = ITEM(nrows);
+#undef ITEM
+      const int e_gr = t * kTileM + rho;   // row of the item
+      const bool e_valid = e_gr < e_nrows;
+      const int e_row = e_row0 + e_gr, e_tok = e_valid ? e_row / p.G : 0;
+      const int64_t oi = (int64_t)(q_start + e_tok) * p.n_q_heads + kv_head * p.G + (e_valid ? e_row % p.G : 0);
       // ---- epilogue: normalise, store
-      const bool live = m_ref != kNegInf && l_sum > 0.f;   // a row with no allowed position: O = 0, LSE = -inf
-      const float inv = live ? 1.f / l_sum : 0.f;
-      const float lse = live ? (m_ref + log2f(l_sum)) * kLn2 : kNegInf;
       // A full tile of final rows leaves through shared memory: every thread converts its row, 64 columns at a
-      // time, into the warpgroup's staging slab (the swizzled image of the box 64 dims x G heads x 128 / G tokens
+      // time, into the Q tile's staging slab (the swizzled image of the box 64 dims x G heads x 128 / G tokens
       // of the output tensor) and one thread hands the slab to a TMA store.  The accumulator is free for the next
       // item as soon as it has been read into registers, and the stores to global memory run while the warpgroup
       // is already in the next item's softmax - the epilogue sits between the last MMA of an item and the first
       // of the next, so every cycle of it is idle tensor-pipe time.  (All conditions are uniform over the
-      // warpgroup: the barriers below always see their 128 threads.)
-      const bool via_tma = use_omap && nhalf > 0 && item.partial_slot < 0 && item.nrows >= (t + 1) * kTileM;
+      // warpgroups of a Q tile: the barriers below always see all their threads.)
+      const bool via_tma = use_omap && nhalf > 0 && partial_slot < 0 && e_nrows >= (t + 1) * kTileM;
+      const bool lead = (warp & 3) == 0 && hw == 0;
+      auto sync_tile = [&]() {   // the 128 (SPLIT: 256) threads of the Q tile
+        if (t == 0) wg_sync<1, C::NWG / 2 * 128>();
+        else wg_sync<2, C::NWG / 2 * 128>();
+      };
+      // SPLIT: both warpgroups of a Q tile scale the two accumulators to the larger reference and take half of the
+      // columns each.  The scales are known before the accumulators are.  (Two buffers: a warpgroup may write its pair of the
+      // next item while the other one still reads.)
+      float f_a = 1.f, f_b = 0.f;
+      if (C::SPLIT && nhalf > 0) {
+        float2* ml = sML + (my_items & 1) * 4 * kTileM + 2 * t * kTileM + rho;
+        ml[hw * kTileM] = make_float2(m_ref, l_sum);
+        if (via_tma && lead) {   // the slab's previous store must have read it before it is overwritten
+          if (elect_one()) bulk_wait_read();
+          __syncwarp();
+        }
+        sync_tile();
+        const float2 a = ml[0], b = ml[kTileM];
+        m_ref = fmaxf(a.x, b.x);
+        f_a = a.x == kNegInf ? 0.f : fast_exp2(a.x - m_ref);
+        f_b = b.x == kNegInf ? 0.f : fast_exp2(b.x - m_ref);
+        l_sum = a.y * f_a + b.y * f_b;
+      }
+      const bool live = m_ref != kNegInf && l_sum > 0.f;   // a row with no allowed position: O = 0, LSE = -inf
+      const float inv = live ? 1.f / l_sum : 0.f;
+      const float lse = live ? (m_ref + log2f(l_sum)) * kLn2 : kNegInf;
+      const bool two = C::SPLIT && nhalf > 1;   // (an item of one half has no second accumulator)
+      f_a *= inv, f_b *= inv;
+      if (nhalf > 0) {
+        mbar_wait(smem_u32(o_done + t), my_items & 1, p.status);
+        ++my_items;
+        tc_fence_after();
+      }
+      constexpr int kStep = C::SPLIT ? 16 : 32;
+      auto read_cols = [&](int c0, float* v) {   // kStep normalised columns of the row
+        if constexpr (C::SPLIT) {
+          const uint32_t tA = tmem + 256 + 2 * t * D + lane_sel + c0;
+          uint32_t ob[kStep];
+          tmem_ld16(tA, reinterpret_cast<uint32_t*>(v));
+          tmem_ld16(tA + (two ? D : 0), ob);
+          tmem_wait_ld();
+#pragma unroll
+          for (int c = 0; c < kStep; ++c) {
+            v[c] = fmaf(two ? __uint_as_float(ob[c]) : 0.f, f_b, v[c] * f_a);
+          }
+        } else {
+          tmem_ld32(tO + c0, reinterpret_cast<uint32_t*>(v));
+          tmem_wait_ld();
+#pragma unroll
+          for (int c = 0; c < kStep; ++c) v[c] *= inv;
+        }
+      };
+      constexpr int kCols = C::SPLIT ? D / 2 : D;   // columns of this warpgroup, from col0 on
+      const int col0 = C::SPLIT ? hw * kCols : 0;
       if (via_tma) {
         const uint32_t stg = smem_u32(sO + t * C::OSLAB) + rho * 128;
-        const bool lead = (warp & 3) == 0;
-        const int tok0 = item.q_start + (item.row0 + t * kTileM) / p.G;
-        auto sync_wg = [&]() {
-          if (t == 0) wg_sync<1>();
-          else wg_sync<2>();
-        };
+        const int tok0 = q_start + (e_row0 + t * kTileM) / p.G;
 #pragma unroll
-        for (int c0 = 0; c0 < D; c0 += 32) {
-          uint32_t o[32];
-          tmem_ld32(tO + c0, o);
-          tmem_wait_ld();
-          if (c0 + 32 == D) {   // O_t is in registers: the next item's PV may overwrite it
+        for (int cc = 0; cc < kCols; cc += kStep) {
+          const int c0 = col0 + cc;
+          float v[kStep];
+          read_cols(c0, v);
+          if (cc + kStep == kCols) {   // O_t is in registers: the next item's PV may overwrite it
             tc_fence_before();
             mbar_arrive(smem_u32(o_free + t));
           }
-          uint32_t w[16];
+          uint32_t w[kStep / 2];
 #pragma unroll
-          for (int c = 0; c < 32; c += 2) w[c >> 1] = pack_bf16(__uint_as_float(o[c]) * inv, __uint_as_float(o[c + 1]) * inv);
-          if ((c0 & 63) == 0) {   // the slab's previous store must have read it before it is overwritten
+          for (int c = 0; c < kStep; c += 2) w[c >> 1] = pack_bf16(v[c], v[c + 1]);
+          if (!C::SPLIT && (cc & 63) == 0) {   // the slab's previous store must have read it before it is overwritten
             if (lead) {
               if (elect_one()) bulk_wait_read();
               __syncwarp();
             }
-            sync_wg();
+            sync_tile();
           }
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
+          for (int k = 0; k < kStep / 8; ++k) {
             const int ch = ((c0 & 63) >> 3) + k;   // 16-byte chunk of the row inside the slab
             st_shared_v4(stg + ((ch ^ (rho & 7)) << 4), w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
           }
-          if ((c0 & 63) == 32) {
+          if (C::SPLIT ? cc + kStep == kCols : (cc & 63) == 32) {
             fence_async_smem();
-            sync_wg();
+            sync_tile();
             if (lead) {
               if (elect_one()) {
-                tma_store_3d(&omap, smem_u32(sO + t * C::OSLAB), c0 & ~63, item.kv_head * p.G, tok0);
+                tma_store_3d(&omap, smem_u32(sO + t * C::OSLAB), c0 & ~63, kv_head * p.G, tok0);
                 bulk_commit();
               }
               __syncwarp();
             }
           }
         }
-        p.lse[oi] = lse;
+        if (hw == 0) p.lse[oi] = lse;
       } else {
 #pragma unroll
-        for (int c0 = 0; c0 < D; c0 += 32) {
-          uint32_t o[32];
+        for (int cc = 0; cc < kCols; cc += kStep) {
+          const int c0 = col0 + cc;
+          float v[kStep];
           if (nhalf > 0) {
-            tmem_ld32(tO + c0, o);
-            tmem_wait_ld();
+            read_cols(c0, v);
           } else {
 #pragma unroll
-            for (int c = 0; c < 32; ++c) o[c] = 0u;
+            for (int c = 0; c < kStep; ++c) v[c] = 0.f;
           }
-          if (valid) {
-            if (item.partial_slot < 0) {
+          if (e_valid) {
+            if (partial_slot < 0) {
               // 32-byte stores: every thread writes its own row, so the store path is bound by the number
               // of (thread, instruction) pairs, not by bytes
               __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.out) + oi * D + c0;
-              uint32_t w[16];
+              uint32_t w[kStep / 2];
 #pragma unroll
-              for (int c = 0; c < 32; c += 2) w[c >> 1] = pack_bf16(__uint_as_float(o[c]) * inv, __uint_as_float(o[c + 1]) * inv);
+              for (int c = 0; c < kStep; c += 2) w[c >> 1] = pack_bf16(v[c], v[c + 1]);
               if (out_wide) {
-                st_global_v8(dst, w);
-                st_global_v8(dst + 16, w + 8);
+#pragma unroll
+                for (int c = 0; c < kStep / 2; c += 8) st_global_v8(dst + 2 * c, w + c);
               } else {
 #pragma unroll
-                for (int c = 0; c < 16; c += 4) reinterpret_cast<uint4*>(dst)[c >> 2] = make_uint4(w[c], w[c + 1], w[c + 2], w[c + 3]);
+                for (int c = 0; c < kStep / 2; c += 4) reinterpret_cast<uint4*>(dst)[c >> 2] = make_uint4(w[c], w[c + 1], w[c + 2], w[c + 3]);
               }
             } else {
-              float* dst = p.ws_o + ((int64_t)item.partial_slot * 256 + (gr - item.row0)) * D + c0;
+              float* dst = p.ws_o + ((int64_t)partial_slot * 256 + e_gr) * D + c0;
 #pragma unroll
-              for (int c = 0; c < 32; c += 8) {
+              for (int c = 0; c < kStep; c += 8) {
                 uint32_t w[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) w[k] = __float_as_uint(__uint_as_float(o[c + k]) * inv);
+                for (int k = 0; k < 8; ++k) w[k] = __float_as_uint(v[c + k]);
                 st_global_v8(dst + c, w);
               }
             }
           }
         }
-        if (valid) {
-          if (item.partial_slot < 0) p.lse[oi] = lse;
-          else p.ws_lse[(int64_t)item.partial_slot * 256 + (gr - item.row0)] = lse;
+        if (e_valid && hw == 0) {
+          if (partial_slot < 0) p.lse[oi] = lse;
+          else p.ws_lse[(int64_t)partial_slot * 256 + e_gr] = lse;
         }
         if (nhalf > 0) {
           tc_fence_before();
@@ -844,7 +916,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const AttnParams p
   if (p.late_trigger) pie_pdl_launch_dependents();
   tc_fence_before();
   __syncthreads();
-  if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+  if (warp == kProducer) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }
 
 }  // namespace
@@ -899,7 +971,7 @@ static int launch_tc(pie_ctx* ctx, const AttnParams& p, int grid, int64_t n_toke
   memset(&omap, 0, sizeof(omap));
   const int kflags = (make_q_map(ctx, p.q, n_tokens, p.G, &qmap) ? 1 : 0) | ((reinterpret_cast<uintptr_t>(p.out) & 31) == 0 ? 2 : 0) |
                      (make_q_map(ctx, p.out, n_tokens, p.G, &omap) ? 4 : 0);
-  PIE_CUDA(ctx, pie_launch_pdl(kern, dim3(grid), dim3(kThreads), C::SMEM, s, p, qmap, omap, kflags));
+  PIE_CUDA(ctx, pie_launch_pdl(kern, dim3(grid), dim3(C::THREADS), C::SMEM, s, p, qmap, omap, kflags));
   return PIE_OK;
 }
 
