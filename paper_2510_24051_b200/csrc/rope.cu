@@ -46,24 +46,23 @@ struct Vec16<float> {
   __device__ static void store(void* p, const float* f) { *reinterpret_cast<float4*>(p) = make_float4(f[0], f[1], f[2], f[3]); }
 };
 
-// A block rotates the rows [row_begin, row_end) of 256 / (D / 2) tokens; a token's rows are its query heads (rotated into
+// A block rotates the rows [row_begin, row_end) of THREADS / (D / 2) tokens; a token's rows are its query heads (rotated into
 // qrot), its new K rows (rotated into the pool) and its new V rows (copied into the pool).  Sines and cosines depend on
 // (token, pair) only: every thread makes ONE of them (fp64 angle, sincosf) - before it waits for the kernels in front -,
 // and a thread's pairs (one 16-byte chunk of the first half of a row and its partner in the second half) stay in registers
 // while it walks over the rows of its token.  With a sine and cosine per element of every head the kernel was bound by
 // that arithmetic: five prompts of 7,560 tokens in all, 32 / 8 heads of 64: 129.7 us per step then, 125.1 now.
-constexpr int kRopeThreads = 256;
-template <typename T, int D>
-__global__ void __launch_bounds__(kRopeThreads) rope_kernel(uint8_t* __restrict__ pool, const uint8_t* __restrict__ q, uint8_t* __restrict__ qrot,
+template <typename T, int D, int THREADS>
+__global__ void __launch_bounds__(THREADS) rope_kernel(uint8_t* __restrict__ pool, const uint8_t* __restrict__ q, uint8_t* __restrict__ qrot,
                                                             const uint8_t* __restrict__ k_new, const uint8_t* __restrict__ v_new,
                                                             const int32_t* __restrict__ append_dst, const int32_t* __restrict__ positions,
                                                             const double* __restrict__ inv_freq, int Tn, int n_q_heads, int rows_per_block, PoolGeom g) {
   constexpr int N = Vec16<T>::N;
-  constexpr int HALF = D / 2, TOKENS = kRopeThreads / HALF;
+  constexpr int HALF = D / 2, TOKENS = THREADS / HALF;
   constexpr int HC = HALF / N;                              // 16-byte chunks in half a row
-  constexpr int GROUPS = kRopeThreads / (HC * TOKENS);      // threads with the same token and chunk: they share its rows
+  constexpr int GROUPS = THREADS / (HC * TOKENS);      // threads with the same token and chunk: they share its rows
   constexpr int ROW = D * (int)sizeof(T);
-  __shared__ float2 table[TOKENS][HALF];
+  __shared__ float2 table[TOKENS][HALF + 2];                // (+ 2: the tokens of a warp read different banks)
   pie_pdl_launch_dependents();
   const int t0 = blockIdx.x * TOKENS;
   {
@@ -124,14 +123,14 @@ __global__ void __launch_bounds__(kRopeThreads) rope_kernel(uint8_t* __restrict_
   }
 }
 
-template <typename T, int D>
+template <typename T, int D, int THREADS>
 int launch_rope(pie_ctx* ctx, const pie_plan* plan, const void* q, const void* k_new, const void* v_new, cudaStream_t s) {
-  constexpr int TOKENS = kRopeThreads / (D / 2), GROUPS = kRopeThreads / (D / 2 / Vec16<T>::N * TOKENS);
+  constexpr int TOKENS = THREADS / (D / 2), GROUPS = THREADS / (D / 2 / Vec16<T>::N * TOKENS);
   const int blocks = (plan->T + TOKENS - 1) / TOKENS, rows = ctx->cfg.num_q_heads + 2 * ctx->geom.n_kv_heads;
   // a token's rows over several blocks while there are SMs without one (at least one row per thread)
   const int parts = std::max(1, std::min((2 * ctx->n_sms + blocks - 1) / blocks, (rows + GROUPS - 1) / GROUPS));
   const int rows_per_block = (rows + parts - 1) / parts;
-  PIE_CUDA(ctx, pie_launch_pdl(rope_kernel<T, D>, dim3(blocks, (rows + rows_per_block - 1) / rows_per_block), dim3(kRopeThreads), 0, s, ctx->pool,
+  PIE_CUDA(ctx, pie_launch_pdl(rope_kernel<T, D, THREADS>, dim3(blocks, (rows + rows_per_block - 1) / rows_per_block), dim3(THREADS), 0, s, ctx->pool,
                                (const uint8_t*)q, (uint8_t*)ctx->d_qrot, (const uint8_t*)k_new, (const uint8_t*)v_new,
                                (const int32_t*)plan->d_append_dst, (const int32_t*)plan->d_positions, (const double*)ctx->d_inv_freq, plan->T,
                                ctx->cfg.num_q_heads, rows_per_block, ctx->geom));
@@ -143,7 +142,13 @@ int launch_rope(pie_ctx* ctx, const pie_plan* plan, const void* q, const void* k
 int pie_launch_rope(pie_ctx* ctx, const pie_plan* plan, const void* q, const void* k_new, const void* v_new, cudaStream_t s) {
   if (plan->T == 0) return PIE_OK;
   const bool bf16 = ctx->cfg.dtype == PIE_DTYPE_BF16;
+  // bf16 batches that fill the chip: blocks of 128 threads, whose loads, arithmetic and stores mix better on an SM than those
+  // of 256 (five prompts of 7,560 tokens 121.2 -> 118.9 us per step).  Smaller ones, where a token's rows are spread over
+  // blocks that each make its sines and cosines again, and fp32 rows lose with them (120 decodes 309.7 -> 311.2 us, five
+  // short fp32 prompts 63.1 -> 65.7 us).
+  if (!bf16) return ctx->cfg.head_dim == 64 ? launch_rope<float, 64, 256>(ctx, plan, q, k_new, v_new, s) : launch_rope<float, 128, 256>(ctx, plan, q, k_new, v_new, s);
+  const bool fills = (int64_t)plan->T * ctx->cfg.head_dim >= (int64_t)2 * 512 * ctx->n_sms;   // two blocks of 256 threads per SM
   if (ctx->cfg.head_dim == 64)
-    return bf16 ? launch_rope<__nv_bfloat16, 64>(ctx, plan, q, k_new, v_new, s) : launch_rope<float, 64>(ctx, plan, q, k_new, v_new, s);
-  return bf16 ? launch_rope<__nv_bfloat16, 128>(ctx, plan, q, k_new, v_new, s) : launch_rope<float, 128>(ctx, plan, q, k_new, v_new, s);
+    return fills ? launch_rope<__nv_bfloat16, 64, 128>(ctx, plan, q, k_new, v_new, s) : launch_rope<__nv_bfloat16, 64, 256>(ctx, plan, q, k_new, v_new, s);
+  return fills ? launch_rope<__nv_bfloat16, 128, 128>(ctx, plan, q, k_new, v_new, s) : launch_rope<__nv_bfloat16, 128, 256>(ctx, plan, q, k_new, v_new, s);
 }
