@@ -1454,7 +1454,8 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
       }
     }
   }
-  // split-KV decode.  Long launches: chunks taken dynamically by the warps of the grid (evens out
+  // split-KV decode.  Plain launches: a block or a cluster of blocks per unit (pick_cluster).  The others - cascades, mixed
+  // batches side by side, long launches on 8-token pages, options -:  long ones take chunks dynamically by the warps of the grid (evens out
   // SMs that get different shares of the memory bandwidth: 5-10 % of the launch).  Shorter ones: fixed
   // shares - whole units per thread block with the merge inside the block when that balances, else one
   // equal share per warp and the merge launch.  The dynamic list always needs the merge launch
