@@ -11,8 +11,8 @@
 //                    its own, that meet in the epilogue.  There the exponentials bound the kernel (2,048 cycles per KV tile
 //                    of the two Q tiles at 16 per cycle and SM, the MMAs half of that), and two warps per scheduler left
 //                    that pipe idle in the waits of each half: 2,900 cycles per KV tile; four take 2,500.  us per launch,
-//                    32 / 8 heads, before -> now: 8 chunks of 512 behind 4,096 135 -> 122, 40 behind 2,048 368 -> 337, two
-//                    prompts of 4,000 201 -> 185, 37 chunks of 64 behind 8,000 117 -> 106.  (128-wide heads fill TMEM with two.)
+//                    32 / 8 heads, before -> now: 8 chunks of 512 behind 4,096 135 -> 117, 40 behind 2,048 368 -> 328, two
+//                    prompts of 4,000 201 -> 177, 37 chunks of 64 behind 8,000 117 -> 103.  (128-wide heads fill TMEM with two.)
 //   producer         linear bulk copies of page blocks into the K / V stage rings.  The
 //                    pool's storage order is the 128-byte-swizzled canonical operand layout, so a
 //                    page block drops into its 16-row band of the tile with no tensor map.
@@ -152,6 +152,28 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
   uint64_t r;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
+}
+// 2^y for a pair on the FMA pipe: y = n + r with r in [-0.5, 0.5] (n by adding and subtracting 1.5 * 2^23), 2^r as the
+// polynomial of degree 5 with the smallest largest relative error there (Remez exchange in fp64; 1.8 * 2^-23 with its fp32
+// rounding, ex2.approx has 2 * 2^-23), n added to the exponent.  y is clamped to [-126, 126].
+__device__ __forceinline__ void exp2_poly(uint64_t y2, float& e0, float& e1) {
+  float y0, y1;
+  unpack_f32x2(y2, y0, y1);
+  y2 = pack_f32x2(fminf(fmaxf(y0, -126.f), 126.f), fminf(fmaxf(y1, -126.f), 126.f));
+  const uint64_t z2 = add_f32x2(y2, pack_f32x2(12582912.f, 12582912.f));
+  const uint64_t n2 = add_f32x2(z2, pack_f32x2(-12582912.f, -12582912.f));
+  const uint64_t r2 = fma_f32x2(n2, pack_f32x2(-1.f, -1.f), y2);
+  auto k = [](float c) { return pack_f32x2(c, c); };
+  uint64_t q2 = fma_f32x2(r2, k(0.0013276471992533984f), k(0.009675541334453752f));
+  q2 = fma_f32x2(q2, r2, k(0.055507132734978495f));
+  q2 = fma_f32x2(q2, r2, k(0.24022119723839974f));
+  q2 = fma_f32x2(q2, r2, k(0.6931469670647609f));
+  q2 = fma_f32x2(q2, r2, k(1.0000000716546849f));
+  float z0, z1, q0, q1;
+  unpack_f32x2(z2, z0, z1);
+  unpack_f32x2(q2, q0, q1);
+  e0 = __uint_as_float(__float_as_uint(q0) + (__float_as_uint(z0) << 23));   // (the low bits of z hold n)
+  e1 = __uint_as_float(__float_as_uint(q1) + (__float_as_uint(z1) << 23));
 }
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float r;
@@ -603,13 +625,22 @@ __global__ void __launch_bounds__(TcCfg<D, P>::THREADS, 1) attn_tc_kernel(const 
         if (clean_halves <= 1) load_recs(half_of(1), rec_nxt);
 
         // P = exp2(x * scale - m) for one chunk of 32 columns: bf16 pairs into pk, the sums onto sa / sb.
-        auto exp_chunk = [&](const float* x, const uint64_t scale2, const uint64_t negm2, uint64_t& sa, uint64_t& sb, uint32_t* pk) {
+        // SPLIT, lean copy: two of the 16 pairs go to the FMA pipe - the exponential pipe is 81 % busy there and the schedulers
+        // 40 % (8 chunks of 512 behind 4,096: 122.5 us without, 117.1 so, 122 with four pairs, 141 with half of them; with
+        // 8-token pages 138.3 without, 144 so).
+        auto exp_chunk = [&](const float* x, const uint64_t scale2, const uint64_t negm2, uint64_t& sa, uint64_t& sb, uint32_t* pk, auto poly_tag) {
 #pragma unroll
           for (int c = 0; c < 32; c += 4) {
-            float e0, e1, e2, e3;
-            unpack_f32x2(fma_f32x2(pack_f32x2(x[c], x[c + 1]), scale2, negm2), e0, e1);
+            float e0, e1, e2, e3, p0, p1;
+            const uint64_t y2 = fma_f32x2(pack_f32x2(x[c], x[c + 1]), scale2, negm2);
             unpack_f32x2(fma_f32x2(pack_f32x2(x[c + 2], x[c + 3]), scale2, negm2), e2, e3);
-            const float p0 = fast_exp2(e0), p1 = fast_exp2(e1), p2 = fast_exp2(e2), p3 = fast_exp2(e3);
+            if (decltype(poly_tag)::value && c % 16 == 0) {
+              exp2_poly(y2, p0, p1);
+            } else {
+              unpack_f32x2(y2, e0, e1);
+              p0 = fast_exp2(e0), p1 = fast_exp2(e1);
+            }
+            const float p2 = fast_exp2(e2), p3 = fast_exp2(e3);
             sa = add_f32x2(sa, pack_f32x2(p0, p1));
             sb = add_f32x2(sb, pack_f32x2(p2, p3));
             pk[c >> 1] = pack_bf16(p0, p1);
@@ -668,7 +699,7 @@ __global__ void __launch_bounds__(TcCfg<D, P>::THREADS, 1) attn_tc_kernel(const 
                 const uint64_t negm2 = pack_f32x2(-m_ref, -m_ref);
                 uint64_t ca = pack_f32x2(0.f, 0.f), cb = pack_f32x2(0.f, 0.f);
                 uint32_t pk[16];
-                exp_chunk(x, scale2, negm2, ca, cb, pk);
+                exp_chunk(x, scale2, negm2, ca, cb, pk, std::integral_constant<bool, !kMasked && C::SPLIT && P != 8>{});
                 float s0, s1;
                 unpack_f32x2(add_f32x2(ca, cb), s0, s1);
                 if (!__any_sync(0xFFFFFFFFu, !(s0 + s1 <= 65536.f))) {   // (also catches inf and NaN)
@@ -730,7 +761,7 @@ __global__ void __launch_bounds__(TcCfg<D, P>::THREADS, 1) attn_tc_kernel(const 
             const uint64_t negm2 = pack_f32x2(neg_m, neg_m);
             uint64_t ca = pack_f32x2(0.f, 0.f), cb = pack_f32x2(0.f, 0.f);
             uint32_t pk[16];
-            exp_chunk(x, scale2, negm2, ca, cb, pk);
+            exp_chunk(x, scale2, negm2, ca, cb, pk, std::false_type{});
             float s0, s1;
             unpack_f32x2(add_f32x2(ca, cb), s0, s1);
             l_sum += s0 + s1;
