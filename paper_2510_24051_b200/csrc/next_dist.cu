@@ -5,25 +5,29 @@
 // owns a contiguous part of the row and
 //   1. reads it once, 16 bytes per load, up to NG loads in flight per thread: running maxima (several per thread, of
 //      disjoint subsets of its entries) and the sum of exponentials relative to the thread's maximum;
-//   2. builds a histogram of those subset maxima by the upper 16 bits of their order-preserving key and takes the bin
-//      that holds the ceil(K / S)-th largest: the smallest of the blocks' bins is tau.  At least K entries of the row
-//      lie at or above tau (that many subset maxima alone), so nothing below it can be part of the answer, and few
-//      more than K entries pass;
+//   2. builds a histogram of those subset maxima by the upper 16 bits of their order-preserving key - a bin each for the 1,024
+//      below the block's maximum (8 binades), one per half binade beyond - and takes the bin that holds the ceil(K / S)-th
+//      largest: the lower end of the smallest of the blocks' bins is tau.  At least K entries of the row lie at or above tau
+//      (that many subset maxima alone), so nothing below it can be part of the answer, and few more than K entries pass;
 //   3. collects its entries at or above tau - from registers when the part was NG groups per thread, else from L2 - and
 //      copies them into the pool of block 0 through distributed shared memory.
-// Block 0 sorts the few hundred candidates by counting (bin = upper 16 bits of the key; inside a bin by logit and
-// ascending token id) and writes the first K with their probabilities exp(x - max) / sum, not renormalised.
-// Rows with so many equal entries around the K-th place that more than 4,096 entries pass (quantised logits,
-// constant rows) are redone by block 0 the general way: radix selection of the K-th largest key, eight bits per pass.
+// When some block has fewer maxima than that (a part of the row that is masked out), or its bin holds most of them (fp32 logits
+// with a large common offset, log-probabilities with a confident top), tau is the K-th largest of ALL blocks' subset maxima
+// instead (union_threshold), and step 3 follows with that.
+// Block 0 sorts the few hundred candidates by counting (bin = leading bits of the key's distance from the maximum's; inside a bin
+// by logit and ascending token id) and writes the first K with their probabilities exp(x - max) / sum, not renormalised.
+// Rows of which more than 4,096 entries reach tau (constant rows, very many equal entries at the K-th place) are left to block 0
+// alone: radix selection of the K-th largest key, eight bits per pass.
 //
 // Bound: a chain of latencies (launch, one read, four block barriers, two cluster barriers, the sort) for decode-sized batches,
-// the exponential unit and issue slots (about 50 instructions per 8 bf16 entries) for hundreds of rows.  Two blocks of 512
-// threads share an SM, so that one block's chain hides behind another's stream.  Measured (captured graphs, K = 256, us per call;
-// in brackets the kernels this one replaced, one block or one cluster of 1,024 threads per row and SM):
-//   bf16  1 x 128,256  7.3 (10.5)   64 x 128,256  12.9 (13.7)   64 x 50,257  10.2 (25.1)   512 x 8,000  18.2 (127)   512 x 128,256  79 (92)
-//   fp32  1 x 128,256  7.6 (23.8)   64 x 128,256  14.8 (25.5)   512 x 128,256  90 (113)
-// Many long rows stay far from the HBM time (20 us for 512 x 128,256 bf16): 147 instructions per 8 entries and group, and
-// instruction fetch, not data, is the first stall.
+// the exponential unit, issue slots and instruction fetch for hundreds of rows.  Two blocks of 512 threads share an SM, so that
+// one block's chain hides behind another's stream.
+// Measured (captured graphs, centred logits, us per call; in brackets one block, or one cluster, of 1,024 threads per row and SM):
+//   bf16  1 x 128,256, K = 256  7.5 (10.5)   64 x 128,256  12.9 (13.5)   64 x 50,257  10.1 (25)   512 x 8,000  18.4 (125)   512 x 128,256  77 (92)
+//   fp32  1 x 128,256  7.1 (22)   64 x 128,256  13.3 (25)   512 x 128,256  87 (114)
+// 64 x 128,256 with a positive maximum over a negative K-th logit 13.6 / 14.2 (204 / 334 while the histogram ended 16 binades below the
+// maximum and such rows passed whole), log-probabilities with a confident top 24 / 25 (364 / 477), the second half masked out 21 / 22,
+// constant rows 133 / 226.  Many long rows stay far from the HBM time (20 us for 512 x 128,256 bf16).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -41,9 +45,11 @@ constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxK = 1024;
 constexpr int kMaxCand = 4096;   // entries the filter may pass before the radix path takes over
-constexpr int kBins = 2048;      // upper-16-bit keys below the maximum that histogram and counting sort tell apart
+constexpr int kBins = 2048;      // of the histograms and of the counting sort
 constexpr uint32_t kMaxBin = 512;   // candidates of one bin that are ranked by comparing all pairs (1 - 4 us; sorting 2,048 candidates takes 18 us)
 constexpr int kMaxCluster = 8;
+constexpr uint32_t kFiniteKey = 0x00800000u;   // of -FLT_MAX, and not above that of the lowest finite bf16 value
+constexpr uint32_t kFine = 1024;   // bins of one upper-16-bit key each below the maximum; the others hold 64 (kFine + (65536 - kFine) / 64 <= kBins)
 static_assert(kMaxCand * 8 >= kWarps * 256 * 4, "the histograms fit into the candidate buffer");
 
 // Order-preserving key: larger logit <=> larger unsigned key.  bf16 keys sit in the upper half.
@@ -124,15 +130,6 @@ __device__ __forceinline__ uint32_t entry_bits(const uint32_t* w, int e) {
   if (Elem<T>::VEC == 4) return w[e];
   return (e & 1) ? (w[e >> 1] & 0xFFFF0000u) : (w[e >> 1] << 16);
 }
-template <typename T>
-__device__ __forceinline__ void load_keys(const T* __restrict__ row, int vocab, const RowGrid& rg, int g, uint32_t* keys) {
-  uint4 v = make_uint4(Elem<T>::NEG_INF2, Elem<T>::NEG_INF2, Elem<T>::NEG_INF2, Elem<T>::NEG_INF2);
-  if (g < rg.n_groups) v = load_group<T>(row, vocab, rg, g);
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int e = 0; e < Elem<T>::VEC; ++e) keys[e] = key_of_bits(entry_bits<T>(w, e));
-}
-
 // Bitonic sort of a[0, n) in shared memory, descending; n is a power of two, the whole block takes part.
 __device__ __forceinline__ void sort_descending(unsigned long long* a, int n) {
   for (int size = 2; size <= n; size <<= 1) {
@@ -154,35 +151,64 @@ __device__ __forceinline__ void sort_descending(unsigned long long* a, int n) {
 struct NdScratch {
   unsigned long long pool[kMaxCand];   // block 0: candidates of the whole row (key << 32 | ~token id); the radix path keeps its histograms here
   unsigned long long cand[kMaxCand];   // this block's candidates; then, in block 0, all candidates grouped by bin; the K survivors of the radix path
+  uint32_t ranges[2][kWarps];          // union_threshold: totals of the histograms' ranges
   uint32_t bin_start[kBins], bin_cur[kBins];
   float red[kWarps];
   uint32_t scan[kWarps];
   uint32_t x_lo[kMaxCluster], x_hi[kMaxCluster];   // every block's threshold / largest key (written by the peers)
   float x_sum[kMaxCluster];                        // block 0: partial sums, each relative to its block's maximum
-  uint32_t sh_prefix, sh_krem, sh_cnt, l_cnt, l_base;
-  float sh_max, sh_sum;
+  uint32_t sh_prefix, sh_krem, sh_stop, sh_cnt, l_cnt, l_base;
 };
 
-// The general way for rows with many equal entries around the K-th place: radix selection of the K-th largest
-// key, eight bits per pass (the first pass also finds the row maximum, the second the sum of exp(x - max) over
-// the whole row), then the entries above it and, in ascending token order, as many entries equal to it as are
-// still missing.  The whole block takes part; reads the row from global memory.
 template <typename T>
-__device__ __noinline__ void radix_path(const T* __restrict__ row, int vocab, int K, int64_t row_idx, int32_t* __restrict__ out_ids,
-                                        float* __restrict__ out_probs, NdScratch& sc) {
-  constexpr int VEC = Elem<T>::VEC;
+struct NdArgs {
+  const T* logits;
+  int64_t row_stride;
+  int vocab, K, subsets;
+  int32_t* out_ids;
+  float* out_probs;
+};
+
+// The row's sum of exponentials from the blocks' (in rank order: the result does not depend on timing), and its largest key
+// unless that is known.
+__device__ __forceinline__ float row_sum(int S, const NdScratch& sc, uint32_t& top) {
+  if (top == 0u)
+    for (int r = 0; r < S; ++r) top = max(top, sc.x_hi[r]);
+  float sum = 0.f;
+  for (int r = 0; r < S; ++r) sum += sc.x_sum[r] * exp2f_fast((value_of_key(sc.x_hi[r]) - value_of_key(top)) * kLog2e);
+  return sum;
+}
+
+// The general way for rows with very many equal entries around the K-th place: radix selection of the K-th largest key,
+// eight bits per pass over the entries at or above `tau`, then the entries above it and, in ascending token order, as many
+// entries equal to it as are still missing.  The whole block takes part; reads the row from global memory, four groups in
+// flight per thread (a row is a chain of these reads: one group in flight and the row's maximum and sum found again
+// here took 190 us for 64 constant bf16 rows of 128,256, now 133).
+template <typename T>
+__device__ __forceinline__ void radix_path(const NdArgs<T>& args, uint32_t tau) {
+  extern __shared__ __align__(16) uint8_t nd_smem[];
+  NdScratch& sc = *reinterpret_cast<NdScratch*>(nd_smem);
+  const int S = (int)cooperative_groups::this_cluster().num_blocks(), vocab = args.vocab, K = args.K;
+  const int64_t row_idx = blockIdx.x / S;
+  const T* __restrict__ row = args.logits + row_idx * args.row_stride;
+  constexpr int VEC = Elem<T>::VEC, U = 4;
   unsigned long long* const pool = sc.pool;
   unsigned long long* const cand = sc.cand;
   uint32_t (*hist)[256] = reinterpret_cast<uint32_t (*)[256]>(pool);   // [kWarps][256], one histogram per warp
-  float* const red = sc.red;
   uint32_t* const scan = sc.scan;
   uint32_t& sh_prefix = sc.sh_prefix;
   uint32_t& sh_krem = sc.sh_krem;
   uint32_t& sh_cnt = sc.sh_cnt;
-  float& sh_max = sc.sh_max;
-  float& sh_sum = sc.sh_sum;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const RowGrid rg = row_grid(row, vocab);
+  auto load_groups = [&](int g0, uint4* v) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int g = g0 + u * kThreads + tid;
+      v[u] = make_uint4(Elem<T>::NEG_INF2, Elem<T>::NEG_INF2, Elem<T>::NEG_INF2, Elem<T>::NEG_INF2);
+      if (g < rg.n_groups) v[u] = load_group<T>(row, vocab, rg, g);
+    }
+  };
   __syncthreads();
   if (tid == 0) {
     sh_cnt = 0u;
@@ -190,51 +216,42 @@ __device__ __noinline__ void radix_path(const T* __restrict__ row, int vocab, in
     sh_krem = (uint32_t)K;
   }
 
-  float m_loc = -__builtin_huge_valf(), s_loc = 0.f;
   for (int d = 0; d < Elem<T>::DIGITS; ++d) {
     const int shift = 24 - 8 * d;
     for (int b = tid; b < kWarps * 256; b += kThreads) (&hist[0][0])[b] = 0u;
     __syncthreads();
     const uint32_t prefix = sh_prefix;
     const uint32_t himask = d == 0 ? 0u : (0xFFFFFFFFu << (shift + 8));
-    const float row_max = sh_max;   // (valid from the second pass on)
-    for (int g0 = 0; g0 < rg.n_groups; g0 += kThreads) {   // (every thread walks every group: the warp votes below need whole warps)
-      uint32_t keys[VEC];
-      const int base = (g0 + tid) * VEC - rg.lead;
-      load_keys<T>(row, vocab, rg, g0 + tid, keys);
+    uint32_t last = 0u, run = 0u;
+    for (int g0 = 0; g0 < rg.n_groups; g0 += U * kThreads) {
+      uint4 v[U];
+      load_groups(g0, v);
 #pragma unroll
-      for (int e = 0; e < VEC; ++e) {
-        const bool in_row = (uint32_t)(base + e) < (uint32_t)vocab;
-        if (d == 0 && in_row) m_loc = fmaxf(m_loc, value_of_key(keys[e]));
-        if (d == 1 && in_row) s_loc += expf(value_of_key(keys[e]) - row_max);
-        // entries whose higher digits match take part; equal digits in a warp are counted once
-        const bool take = in_row && ((keys[e] & himask) == prefix);
-        if (!__any_sync(0xFFFFFFFFu, take)) continue;
-        const uint32_t digit = (keys[e] >> shift) & 0xFFu;
-        const uint32_t peers = __match_any_sync(0xFFFFFFFFu, take ? digit : 0x100u + (uint32_t)lane);
-        if (take && lane == __ffs(peers) - 1) atomicAdd(&hist[warp][digit], (uint32_t)__popc(peers));
+      for (int u = 0; u < U; ++u) {
+        const int base = (g0 + u * kThreads + tid) * VEC - rg.lead;
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) {
+          // entries whose higher digits match take part; runs of equal digits are counted in a register
+          const uint32_t key = key_of_bits(entry_bits<T>(&v[u].x, e));
+          if ((uint32_t)(base + e) < (uint32_t)vocab && key >= tau && (key & himask) == prefix) {
+            const uint32_t digit = (key >> shift) & 0xFFu;
+            if (digit != last) {
+              if (run) atomicAdd(&hist[warp][last], run);
+              last = digit;
+              run = 0u;
+            }
+            ++run;
+          }
+        }
       }
     }
-    if (d == 0) {   // row maximum
-      for (int o = 16; o > 0; o >>= 1) m_loc = fmaxf(m_loc, __shfl_xor_sync(0xFFFFFFFFu, m_loc, o));
-      if (lane == 0) red[warp] = m_loc;
-    }
-    if (d == 1) {   // sum of exp(x - max) over the whole row
-      for (int o = 16; o > 0; o >>= 1) s_loc += __shfl_xor_sync(0xFFFFFFFFu, s_loc, o);
-      if (lane == 0) red[warp] = s_loc;
-    }
+    if (run) atomicAdd(&hist[warp][last], run);
     __syncthreads();
     if (tid < 256) {   // combine the warps' histograms
       uint32_t c = 0;
 #pragma unroll 8
       for (int w = 0; w < kWarps; ++w) c += hist[w][tid];
       hist[0][tid] = c;
-    }
-    if (warp == 8 && d <= 1) {
-      float v = red[lane % kWarps];
-      if (d == 1 && lane >= kWarps) v = 0.f;
-      for (int o = 16; o > 0; o >>= 1) v = d == 0 ? fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o)) : v + __shfl_xor_sync(0xFFFFFFFFu, v, o);
-      if (lane == 0) (d == 0 ? sh_max : sh_sum) = v;
     }
     __syncthreads();
     if (warp == 0) {
@@ -266,51 +283,59 @@ __device__ __noinline__ void radix_path(const T* __restrict__ row, int vocab, in
     }
     __syncthreads();
   }
-  static_assert(Elem<T>::DIGITS >= 2, "the second pass is where the sum over the row is taken");
 
   // ---- collect: keys above the threshold, and the first k_rem keys equal to it in token order
   const uint32_t thr = sh_prefix, need_eq = sh_krem, n_gt = (uint32_t)K - need_eq;
   uint32_t eq_before = 0;   // equal keys in the groups already walked (same value in every thread)
-  for (int g0 = 0; g0 < rg.n_groups; g0 += kThreads) {
-    uint32_t keys[VEC];
-    const int base = (g0 + tid) * VEC - rg.lead;
-    load_keys<T>(row, vocab, rg, g0 + tid, keys);
-    auto in_row = [&](int e) { return (uint32_t)(base + e) < (uint32_t)vocab; };
-    uint32_t n_eq = 0;
+  for (int g0 = 0; g0 < rg.n_groups; g0 += U * kThreads) {
+    uint4 v[U];
+    load_groups(g0, v);
 #pragma unroll
-    for (int e = 0; e < VEC; ++e) {
-      if (in_row(e) && (keys[e] & Elem<T>::KEY_MASK) > thr) cand[atomicAdd(&sh_cnt, 1u)] = ((unsigned long long)keys[e] << 32) | (0xFFFFFFFFu - (uint32_t)(base + e));
-      n_eq += (in_row(e) && (keys[e] & Elem<T>::KEY_MASK) == thr) ? 1u : 0u;
-    }
-    if (eq_before < need_eq) {   // (uniform) rank the equal keys of this group in token order: block-wide exclusive scan
-      uint32_t incl = n_eq;
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += up;
-      }
-      if (lane == 31) scan[warp] = incl;
-      __syncthreads();
-      uint32_t warp_base = 0, total = 0;
-      for (int w = 0; w < kWarps; ++w) {
-        const uint32_t c = scan[w];
-        if (w < warp) warp_base += c;
-        total += c;
-      }
-      uint32_t rank = eq_before + warp_base + incl - n_eq;
+    for (int u = 0; u < U; ++u) {
+      const int base = (g0 + u * kThreads + tid) * VEC - rg.lead;
+      uint32_t keys[VEC];
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) keys[e] = key_of_bits(entry_bits<T>(&v[u].x, e));
+      auto in_row = [&](int e) { return (uint32_t)(base + e) < (uint32_t)vocab; };
+      uint32_t n_eq = 0;
 #pragma unroll
       for (int e = 0; e < VEC; ++e) {
-        if (in_row(e) && (keys[e] & Elem<T>::KEY_MASK) == thr) {
-          if (rank < need_eq) cand[n_gt + rank] = ((unsigned long long)keys[e] << 32) | (0xFFFFFFFFu - (uint32_t)(base + e));
-          ++rank;
-        }
+        if (in_row(e) && (keys[e] & Elem<T>::KEY_MASK) > thr)
+          cand[atomicAdd(&sh_cnt, 1u)] = ((unsigned long long)keys[e] << 32) | (0xFFFFFFFFu - (uint32_t)(base + e));
+        n_eq += (in_row(e) && (keys[e] & Elem<T>::KEY_MASK) == thr) ? 1u : 0u;
       }
-      eq_before += total;
-      __syncthreads();   // `scan` is reused by the next group
+      if (eq_before < need_eq) {   // (uniform) rank the equal keys of this group in token order: block-wide exclusive scan
+        uint32_t incl = n_eq;
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+          if (lane >= o) incl += up;
+        }
+        if (lane == 31) scan[warp] = incl;
+        __syncthreads();
+        uint32_t warp_base = 0, total = 0;
+        for (int w = 0; w < kWarps; ++w) {
+          const uint32_t c = scan[w];
+          if (w < warp) warp_base += c;
+          total += c;
+        }
+        uint32_t rank = eq_before + warp_base + incl - n_eq;
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) {
+          if (in_row(e) && (keys[e] & Elem<T>::KEY_MASK) == thr) {
+            if (rank < need_eq) cand[n_gt + rank] = ((unsigned long long)keys[e] << 32) | (0xFFFFFFFFu - (uint32_t)(base + e));
+            ++rank;
+          }
+        }
+        eq_before += total;
+        __syncthreads();   // `scan` is reused by the next group
+      }
     }
   }
   __syncthreads();
 
   // ---- sort the K survivors and write them out
+  uint32_t top = 0u;
+  const float sum = row_sum(S, sc, top);
   int n_sort = 1;
   while (n_sort < K) n_sort <<= 1;
   for (int i = K + tid; i < n_sort; i += kThreads) cand[i] = 0ull;   // padding sorts to the end
@@ -319,8 +344,8 @@ __device__ __noinline__ void radix_path(const T* __restrict__ row, int vocab, in
   for (int i = tid; i < K; i += kThreads) {
     const unsigned long long c = cand[i];
     const float x = value_of_key((uint32_t)(c >> 32));
-    out_ids[row_idx * K + i] = (int32_t)(0xFFFFFFFFu - (uint32_t)c);
-    out_probs[row_idx * K + i] = expf(x - sh_max) / sh_sum;
+    args.out_ids[row_idx * K + i] = (int32_t)(0xFFFFFFFFu - (uint32_t)c);
+    args.out_probs[row_idx * K + i] = expf(x - value_of_key(top)) / sum;
   }
 }
 
@@ -350,11 +375,288 @@ struct SubMax<float> {
   __device__ __forceinline__ float get(int i) const { return m[i]; }
 };
 
+// A key that K of the subset maxima of ALL blocks of the cluster reach and hardly more do - the K-th largest, cut off behind the
+// digit that tells at most 32 of them apart -, or the smallest finite key when fewer than K of them are above -inf: then every
+// finite entry is a candidate.  Leading digits first, 11 bits per round: every block counts its maxima that share the digits
+// found so far, first warps read all blocks' counts through distributed shared memory - the totals of 16 ranges of bins, then
+// the bins of the range that holds the K-th - and all come to the same digit.  (Reading all bins of all blocks in every thread
+// took 5 us a round on 24 rows of 8 blocks.)  The threads' maxima come in `cand`.
+template <typename T>
+__device__ __forceinline__ uint32_t union_threshold(int K, int subsets, NdScratch& sc) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  constexpr int N = SubMax<T>::N, kRange = kBins / kWarps;   // bins per warp
+  static_assert(kBins == 2048 && kRange == 128, "11 bits per round, four bins of a range per lane");
+  const int S = (int)cluster.num_blocks(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const SubMax<T> sub = reinterpret_cast<const SubMax<T>*>(sc.cand)[tid];   // (this thread's own)
+  if (tid == 0) {
+    sc.sh_prefix = sc.sh_stop = 0u;
+    sc.sh_krem = (uint32_t)K;
+  }
+#pragma unroll 1
+  for (int round = 0; round < (N == 8 ? 2 : 3); ++round) {
+    const int shift = round == 0 ? 21 : round == 1 ? 10 : 0;
+    // (what a round writes is read by the peers until they reach the next round's barrier: two buffers of each)
+    uint32_t* hist = round & 1 ? sc.bin_start : sc.bin_cur;
+    uint32_t* ranges = sc.ranges[round & 1];
+    for (int b = tid; b < kBins; b += kThreads) hist[b] = 0u;
+    __syncthreads();
+    const uint32_t prefix = sc.sh_prefix;
+    const uint32_t himask = round == 0 ? 0u : round == 1 ? 0xFFE00000u : 0xFFFFFC00u, digits = round == 2 ? 0x3FFu : 0x7FFu;
+    float x = kNegInf;
+#pragma unroll
+    for (int e = 0; e < N; ++e) {   // `subsets` maxima of N / subsets neighbours each
+      x = fmaxf(x, sub.get(e));
+      if (((e + 1) * subsets) % N == 0) {
+        const uint32_t key = key_of_bits(__float_as_uint(x));
+        if (x != kNegInf && (key & himask) == prefix) atomicAdd(&hist[(key >> shift) & digits], 1u);
+        x = kNegInf;
+      }
+    }
+    __syncthreads();
+    const int b0 = kBins - kRange * (warp + 1) + 4 * (31 - lane);   // range `warp` from the top, its four bins `lane` from the top
+    {
+      const uint4 c = *reinterpret_cast<const uint4*>(&hist[b0]);
+      const uint32_t tot = __reduce_add_sync(0xFFFFFFFFu, c.x + c.y + c.z + c.w);
+      if (lane == 0) ranges[warp] = tot;
+    }
+    cluster.sync();
+    if (warp == 0) {
+      const uint32_t need = sc.sh_krem;
+      auto scan = [&](uint32_t v) {
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, v, o);
+          if (lane >= o) v += up;
+        }
+        return v;
+      };
+      uint32_t tot = 0;
+      for (int r = 0; r < S; ++r) tot += lane < kWarps ? cluster.map_shared_rank(ranges, r)[lane] : 0u;
+      const uint32_t incl = scan(tot);
+      const uint32_t at = __ballot_sync(0xFFFFFFFFu, incl >= need);
+      if (at == 0u) {   // fewer maxima than K (only in the first round, and in every block)
+        if (lane == 0) sc.sh_prefix = kFiniteKey, sc.sh_stop = 1u;
+      } else {
+        const int range = __ffs(at) - 1;
+        const uint32_t before = __shfl_sync(0xFFFFFFFFu, incl - tot, range);
+        const int c0 = kBins - kRange * (range + 1) + 4 * (31 - lane);
+        uint4 c = make_uint4(0u, 0u, 0u, 0u);
+        for (int r = 0; r < S; ++r) {
+          const uint4 y = *reinterpret_cast<const uint4*>(cluster.map_shared_rank(hist, r) + c0);
+          c.x += y.x, c.y += y.y, c.z += y.z, c.w += y.w;
+        }
+        const uint32_t n[4] = {c.w, c.z, c.y, c.x};
+        uint32_t above = before + scan(c.x + c.y + c.z + c.w) - (c.x + c.y + c.z + c.w);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (above < need && need <= above + n[j]) {
+            sc.sh_prefix = prefix | (uint32_t)(c0 + 3 - j) << shift;
+            sc.sh_krem = need - above;
+            sc.sh_stop = n[j] <= 32u ? 1u : 0u;
+          }
+          above += n[j];
+        }
+      }
+    }
+    __syncthreads();
+    if (sc.sh_stop) break;
+  }
+  const uint32_t tau = sc.sh_prefix;
+  cluster.sync();   // (no block clears or leaves counts that a peer still reads)
+  return tau;
+}
+
+// The entries at or above a threshold, into this block's part of the candidates.
+template <typename T>
+struct Filter {
+  float tau_f;
+  uint32_t tau2;
+  __device__ __forceinline__ explicit Filter(uint32_t tau) {
+    tau_f = value_of_key(tau);
+    const uint32_t b = __float_as_uint(tau_f) >> 16;
+    tau2 = b | (b << 16);
+  }
+  static __device__ __forceinline__ void offer(uint32_t bits, int token, int vocab, NdScratch& sc) {
+    if ((uint32_t)token >= (uint32_t)vocab) return;   // (-inf outside the row)
+    const uint32_t at = atomicAdd(&sc.l_cnt, 1u);
+    if (at < (uint32_t)kMaxCand) sc.cand[at] = ((unsigned long long)key_of_bits(bits) << 32) | (0xFFFFFFFFu - (uint32_t)token);
+  }
+  __device__ __forceinline__ void collect(const uint4& x, int token, int vocab, NdScratch& sc) const {
+    const uint32_t* w = &x.x;
+    if constexpr (Elem<T>::VEC == 8) {
+      uint32_t m[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) asm("set.ge.u32.bf16x2 %0, %1, %2;" : "=r"(m[e]) : "r"(w[e]), "r"(tau2));
+      if ((m[0] | m[1] | m[2] | m[3]) != 0u) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if (m[e] & 0x0000FFFFu) offer(w[e] << 16, token + 2 * e, vocab, sc);
+          if (m[e] & 0xFFFF0000u) offer(w[e] & 0xFFFF0000u, token + 2 * e + 1, vocab, sc);
+        }
+      }
+    } else {
+      const float x0 = __uint_as_float(w[0]), x1 = __uint_as_float(w[1]), x2 = __uint_as_float(w[2]), x3 = __uint_as_float(w[3]);
+      if (fmaxf(fmaxf(x0, x1), fmaxf(x2, x3)) >= tau_f) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (__uint_as_float(w[e]) >= tau_f) offer(w[e], token + e, vocab, sc);
+      }
+    }
+  }
+};
+
+// Every block's candidates into the pool of block 0, which has their number in sh_cnt afterwards (all blocks take part).
+__device__ __forceinline__ void gather_candidates(int S, int rank, NdScratch& sc) {
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int tid = threadIdx.x;
+  __syncthreads();
+  const uint32_t n_loc = sc.l_cnt;
+  if (S == 1) {
+    if (tid == 0) sc.sh_cnt = n_loc;
+  } else {
+    if (tid == 0) sc.l_base = atomicAdd(cluster.map_shared_rank(&sc.sh_cnt, 0), n_loc);
+    __syncthreads();
+    const uint32_t base = sc.l_base;
+    unsigned long long* pool0 = cluster.map_shared_rank(&sc.pool[0], 0);
+    for (uint32_t i = tid; i < min(n_loc, (uint32_t)kMaxCand); i += kThreads)
+      if (base + i < (uint32_t)kMaxCand) pool0[base + i] = sc.cand[i];
+  }
+  if (rank == 0)
+    for (int b = tid; b < kBins; b += kThreads) sc.bin_cur[b] = 0u;   // (the histogram is done with: it becomes the counting sort's)
+  cluster.sync();
+}
+
+// Block 0: the candidates in order, the first K written out.  kFew: there may be fewer of them than K.
+template <typename T, bool kFew>
+__device__ __forceinline__ void finish_row(const NdArgs<T>& args, uint32_t tau, uint32_t top, NdScratch& sc) {   // (top = 0: not known yet)
+  const int S = (int)cooperative_groups::this_cluster().num_blocks(), K = args.K;
+  const int64_t row_idx = blockIdx.x / S;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t n_pass = sc.sh_cnt;
+  const float sum = row_sum(S, sc, top);
+  const float row_max_f = value_of_key(top);
+  unsigned long long* src = S == 1 ? sc.cand : sc.pool;
+  unsigned long long* dst = S == 1 ? sc.pool : sc.cand;
+  // bins of the counting sort: distance of the key from the maximum's, as finely as kBins of them reach down to tau.  (bf16 keys
+  // not below the bit that tells them apart: 16 bins from one to the next, they would share two banks.  Equal steps of the logit
+  // instead cost every bf16 row 0.3 us.)
+  const uint32_t span = (top - tau) / (uint32_t)kBins;
+  const int bin_shift = max(Elem<T>::VEC == 8 ? 16 : 0, 32 - __clz(span));
+  auto bin_of = [&](unsigned long long c) { return min((top - (uint32_t)(c >> 32)) >> bin_shift, (uint32_t)kBins - 1u); };
+  auto write_out = [&](unsigned long long c, uint32_t pos) {
+    args.out_ids[row_idx * K + pos] = (int32_t)(0xFFFFFFFFu - (uint32_t)c);
+    args.out_probs[row_idx * K + pos] = expf(value_of_key((uint32_t)(c >> 32)) - row_max_f) / sum;
+  };
+
+  // ---- counting sort: bins in descending order of logit; inside a bin the larger 64-bit value (larger key, then smaller
+  // token id) goes first.
+  uint32_t big = 0u;
+  for (uint32_t i = tid; i < n_pass; i += kThreads)
+    big |= atomicAdd(&sc.bin_cur[bin_of(src[i])], 1u) >= kMaxBin ? 1u : 0u;
+  const int n_out = min(K, (int)n_pass);
+  if (!__syncthreads_or((int)big)) {
+    {   // exclusive scan over the bins: four bins per thread, warp scans, then the warps' totals
+      const uint4 c = *reinterpret_cast<const uint4*>(&sc.bin_cur[4 * tid]);
+      static_assert(kBins == 4 * kThreads, "four bins per thread");
+      const uint32_t tot = c.x + c.y + c.z + c.w;
+      uint32_t incl = tot;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += up;
+      }
+      if (lane == 31) sc.scan[warp] = incl;
+      __syncthreads();
+      uint32_t warp_base = lane < warp ? sc.scan[lane % kWarps] : 0u;
+      warp_base = __reduce_add_sync(0xFFFFFFFFu, warp_base);
+      const uint32_t ex = warp_base + incl - tot;
+      const uint4 st = make_uint4(ex, ex + c.x, ex + c.x + c.y, ex + c.x + c.y + c.z);
+      *reinterpret_cast<uint4*>(&sc.bin_start[4 * tid]) = st;
+      *reinterpret_cast<uint4*>(&sc.bin_cur[4 * tid]) = st;
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < n_pass; i += kThreads) {
+      const unsigned long long c = src[i];
+      dst[atomicAdd(&sc.bin_cur[bin_of(c)], 1u)] = c;   // grouped by bin, any order inside
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < n_pass; i += kThreads) {
+      const unsigned long long mine = dst[i];
+      const uint32_t bin = bin_of(mine);
+      const uint32_t first = sc.bin_start[bin], end = sc.bin_cur[bin];
+      if (first >= (uint32_t)K) continue;
+      uint32_t pos = first;
+      for (uint32_t j = first; j < end; ++j) pos += dst[j] > mine ? 1u : 0u;
+      if (pos < (uint32_t)K) write_out(mine, pos);
+    }
+  } else {   // a bin with very many candidates (equal logits): sort them all
+    int n_sort = 1;
+    while (n_sort < (int)n_pass) n_sort <<= 1;
+    for (int i = (int)n_pass + tid; i < n_sort; i += kThreads) src[i] = 0ull;   // padding sorts to the end
+    __syncthreads();
+    sort_descending(src, n_sort);
+    for (int i = tid; i < n_out; i += kThreads) write_out(src[i], (uint32_t)i);
+  }
+  // ---- fewer finite logits than K (most of the vocabulary masked out): the first of the others in token order.  At most
+  // n_pass of the first K tokens are candidates, so the K - n_pass that are missing are among them.
+  if (kFew && n_out < K) {
+    const T* row = args.logits + row_idx * args.row_stride;
+    const float tau_f = value_of_key(tau);
+    uint32_t place = (uint32_t)n_out;
+    for (int t0 = 0; t0 < K; t0 += kThreads) {
+      const int token = t0 + tid;
+      const uint32_t bits = token < K ? Elem<T>::bits(row + token) : 0u;
+      const bool rest = token < K && !(__uint_as_float(bits) >= tau_f);
+      const uint32_t votes = __ballot_sync(0xFFFFFFFFu, rest);
+      __syncthreads();   // (`scan` is no longer read)
+      if (lane == 0) sc.scan[warp] = (uint32_t)__popc(votes);
+      __syncthreads();
+      const uint32_t part = lane < kWarps ? sc.scan[lane] : 0u;
+      const uint32_t pos = place + __reduce_add_sync(0xFFFFFFFFu, lane < warp ? part : 0u) + (uint32_t)__popc(votes & ((1u << lane) - 1u));
+      if (rest && pos < (uint32_t)K) write_out(((unsigned long long)key_of_bits(bits) << 32) | (0xFFFFFFFFu - (uint32_t)token), pos);
+      place += __reduce_add_sync(0xFFFFFFFFu, part);
+    }
+  }
+}
+
+// The rest of a row for which the common way does not do: histograms that gave no threshold (tau = 0; all blocks of the cluster,
+// the threads' subset maxima in `cand`), or more candidates than block 0 holds (block 0 alone).  A call behind which the kernel ends,
+// everything asked again and the part read again from L2: nothing of it takes registers or instruction cache from the common
+// way.  (Inlined, bf16 rows of centred logits were 8 % slower.)
+template <typename T>
+__device__ __noinline__ void rare_row(const NdArgs<T>& args, uint32_t tau) {
+  if (tau != 0u) {
+    radix_path<T>(args, tau);
+    return;
+  }
+  extern __shared__ __align__(16) uint8_t nd_smem[];
+  NdScratch& sc = *reinterpret_cast<NdScratch*>(nd_smem);
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), tid = threadIdx.x, vocab = args.vocab;
+  const int64_t row_idx = blockIdx.x / S;
+  const T* row = args.logits + row_idx * args.row_stride;
+  const RowGrid rg = row_grid(row, vocab);
+  tau = union_threshold<T>(args.K, args.subsets, sc);
+  const Filter<T> filter(tau);
+  const int per_part = (rg.n_groups + S - 1) / S, g_begin = rank * per_part, g_end = min(rg.n_groups, g_begin + per_part);
+  const int full1 = min(g_end, rg.full1);
+  const uint4* row_groups = reinterpret_cast<const uint4*>(row - rg.lead);
+#pragma unroll 8
+  for (int g = max(g_begin, rg.full0) + tid; g < full1; g += kThreads) filter.collect(__ldg(row_groups + g), g * Elem<T>::VEC - rg.lead, vocab, sc);
+  if (tid < 2) {   // the row's first and last group, where they reach outside the row
+    const int g = tid == 0 ? 0 : rg.n_groups - 1;
+    const bool mine = g >= g_begin && g < g_end && (tid == 0 ? rg.full0 > 0 : rg.full1 < rg.n_groups && rg.n_groups > rg.full0);
+    if (mine) filter.collect(load_group<T>(row, vocab, rg, g), g * Elem<T>::VEC - rg.lead, vocab, sc);
+  }
+  gather_candidates(S, rank, sc);
+  if (rank != 0) return;
+  if (sc.sh_cnt > (uint32_t)kMaxCand) radix_path<T>(args, tau);
+  else finish_row<T, true>(args, tau, 0u, sc);
+}
+
 // NG: loads in flight per thread, and the groups a thread keeps in registers between the two passes.
 template <typename T, int NG>
 __global__ void __launch_bounds__(kThreads, 2)
-next_dist_kernel(const T* __restrict__ logits, int64_t row_stride, int vocab, int K, int subsets, int32_t* __restrict__ out_ids,
-                 float* __restrict__ out_probs) {
+next_dist_kernel(const __grid_constant__ NdArgs<T> args) {
   namespace cg = cooperative_groups;
   constexpr int VEC = Elem<T>::VEC;
   cg::cluster_group cluster = cg::this_cluster();
@@ -363,7 +665,8 @@ next_dist_kernel(const T* __restrict__ logits, int64_t row_stride, int vocab, in
   NdScratch& sc = *reinterpret_cast<NdScratch*>(nd_smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t row_idx = blockIdx.x / S;
-  const T* row = logits + row_idx * row_stride;
+  const int vocab = args.vocab, K = args.K;
+  const T* __restrict__ row = args.logits + row_idx * args.row_stride;
   const RowGrid rg = row_grid(row, vocab);
   const int per_part = (rg.n_groups + S - 1) / S;
   const int g_begin = rank * per_part, g_end = min(rg.n_groups, g_begin + per_part);
@@ -482,12 +785,14 @@ next_dist_kernel(const T* __restrict__ logits, int64_t row_stride, int vocab, in
     if (lane == 0) sc.red[warp] = s;
     // (`subsets` of them: the thread's entries cut into 1, 2, 4 or 8 by their place in the group)
     auto count = [&](float x) {
-      if (x != kNegInf) atomicAdd(&sc.bin_cur[min((hi >> 16) - (key_of_bits(__float_as_uint(x)) >> 16), (uint32_t)kBins - 1u)], 1u);
+      if (x == kNegInf) return;
+      const uint32_t d = (hi >> 16) - (key_of_bits(__float_as_uint(x)) >> 16);
+      atomicAdd(&sc.bin_cur[d < kFine ? d : kFine + ((d - kFine) >> 6)], 1u);
     };
     constexpr int N = SubMax<T>::N;
-    if (subsets == 1) {
+    if (args.subsets == 1) {
       count(m_t);
-    } else if (subsets == 2) {
+    } else if (args.subsets == 2) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         float x = sub.get(h * (N / 2));
@@ -495,7 +800,7 @@ next_dist_kernel(const T* __restrict__ logits, int64_t row_stride, int vocab, in
         for (int i = 1; i < N / 2; ++i) x = fmaxf(x, sub.get(h * (N / 2) + i));
         count(x);
       }
-    } else if (N == 8 && subsets == 4) {
+    } else if (N == 8 && args.subsets == 4) {
 #pragma unroll
       for (int h = 0; h < 4; ++h) count(fmaxf(sub.get(2 * h % N), sub.get((2 * h + 1) % N)));
     } else {
@@ -520,7 +825,7 @@ next_dist_kernel(const T* __restrict__ logits, int64_t row_stride, int vocab, in
     }
     const uint32_t before = incl - tot;
     const uint32_t who = __ballot_sync(0xFFFFFFFFu, before < kb && kb <= incl);
-    uint32_t tau16 = 0u;   // (fewer subset maxima than that, or beyond the bins: every entry passes)
+    uint32_t tau16 = 0u;   // (no threshold)
     if (who) {
       const int l = __ffs(who) - 1;
       const uint32_t run = __shfl_sync(0xFFFFFFFFu, before, l);
@@ -536,7 +841,12 @@ next_dist_kernel(const T* __restrict__ logits, int64_t row_stride, int vocab, in
       const int l2 = __ffs(at) - 1;
       const bool second = __shfl_sync(0xFFFFFFFFu, ex2 + c0, l2) < kb;
       const uint32_t bin = (uint32_t)(l * (kBins / 32) + 2 * l2 + (second ? 1 : 0));
-      if (bin < (uint32_t)kBins - 1u) tau16 = (hi >> 16) - bin;
+      // A fine bin of bf16 is one value.  Others may hold a good part of the row (1/128 of their magnitude wide, the coarse ones half a
+      // binade): with more than 4 kb + 64 maxima, or 7 of 8, at or above its lower end the exact threshold is worth its time.
+      const uint32_t reach = __shfl_sync(0xFFFFFFFFu, second ? run + in2 : ex2 + c0, l2), all = __shfl_sync(0xFFFFFFFFu, incl, 31);
+      const uint32_t d = bin < kFine ? bin : kFine + ((bin - kFine) << 6) + 63u;
+      if ((VEC == 8 && bin < kFine) || vocab <= kMaxK || (reach <= 4u * kb + 64u && 8u * reach <= 7u * all))
+        tau16 = (uint32_t)max((int)(hi >> 16) - (int)d, (int)(kFiniteKey >> 16));
     }
     float s = lane < kWarps ? sc.red[lane] : 0.f;
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
@@ -547,139 +857,36 @@ next_dist_kernel(const T* __restrict__ logits, int64_t row_stride, int vocab, in
     if (lane == 0) *cluster.map_shared_rank(&sc.x_sum[rank], 0) = s;
   }
   cluster.sync();   // (1) every block has every block's threshold and maximum, block 0 the partial sums
-  uint32_t tau16 = 0xFFFFFFFFu, top = 0u;
+  uint32_t tau = 0xFFFFFFFFu, top = 0u;   // (keys; fp32 rows have no register left for `top`)
   for (int r = 0; r < S; ++r) {
-    tau16 = min(tau16, sc.x_lo[r]);
-    top = max(top, sc.x_hi[r]);
+    tau = min(tau, sc.x_lo[r] << 16);
+    if (VEC == 8) top = max(top, sc.x_hi[r]);
   }
-  const float row_max_f = value_of_key(top);
 
   // ---- pass 2: the entries at or above tau, staged in this block, then copied into block 0's pool
-  {
-    const bool all = tau16 == 0u;
-    const float tau_f = value_of_key(tau16 << 16);
-    const uint32_t tau_b = __float_as_uint(tau_f) >> 16, tau2 = tau_b | (tau_b << 16);
-    auto offer = [&](uint32_t bits, int token) {
-      if ((uint32_t)token >= (uint32_t)vocab) return;   // (-inf outside the row)
-      const uint32_t at = atomicAdd(&sc.l_cnt, 1u);
-      if (at < (uint32_t)kMaxCand) sc.cand[at] = ((unsigned long long)key_of_bits(bits) << 32) | (0xFFFFFFFFu - (uint32_t)token);
-    };
-    auto collect = [&](const uint4& x, int token) {
-      const uint32_t* w = &x.x;
-      if constexpr (VEC == 8) {
-        uint32_t m[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) asm("set.ge.u32.bf16x2 %0, %1, %2;" : "=r"(m[e]) : "r"(w[e]), "r"(tau2));
-        if (all) m[0] = m[1] = m[2] = m[3] = 0xFFFFFFFFu;
-        if ((m[0] | m[1] | m[2] | m[3]) != 0u) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            if (m[e] & 0x0000FFFFu) offer(w[e] << 16, token + 2 * e);
-            if (m[e] & 0xFFFF0000u) offer(w[e] & 0xFFFF0000u, token + 2 * e + 1);
-          }
-        }
-      } else {
-        const float x0 = __uint_as_float(w[0]), x1 = __uint_as_float(w[1]), x2 = __uint_as_float(w[2]), x3 = __uint_as_float(w[3]);
-        if (all || fmaxf(fmaxf(x0, x1), fmaxf(x2, x3)) >= tau_f) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (all || __uint_as_float(w[e]) >= tau_f) offer(w[e], token + e);
-        }
-      }
-    };
+  bool rare = tau == 0u;   // (no threshold from the histograms)
+  if (!rare) {
+    const Filter<T> filter(tau);
     for_halves(n_halves <= 2, [&](int h, uint4* x) {
 #pragma unroll
       for (int u = 0; u < H; ++u) {
         const int g = g_begin + (h * H + u) * kThreads + tid;
-        if (g >= rg.full0 && g < min(g_end, rg.full1)) collect(x[u], g * VEC - rg.lead);
+        if (g >= rg.full0 && g < min(g_end, rg.full1)) filter.collect(x[u], g * VEC - rg.lead, vocab, sc);
       }
     });
-    if (edge >= 0) collect(load_group<T>(row, vocab, rg, edge), edge * VEC - rg.lead);
-    __syncthreads();
-    const uint32_t n_loc = sc.l_cnt;
-    if (S == 1) {
-      if (tid == 0) sc.sh_cnt = n_loc;
-    } else {
-      if (tid == 0) sc.l_base = atomicAdd(cluster.map_shared_rank(&sc.sh_cnt, 0), n_loc);
-      __syncthreads();
-      const uint32_t base = sc.l_base;
-      unsigned long long* pool0 = cluster.map_shared_rank(&sc.pool[0], 0);
-      for (uint32_t i = tid; i < min(n_loc, (uint32_t)kMaxCand); i += kThreads)
-        if (base + i < (uint32_t)kMaxCand) pool0[base + i] = sc.cand[i];
-    }
+    if (edge >= 0) filter.collect(load_group<T>(row, vocab, rg, edge), edge * VEC - rg.lead, vocab, sc);
+    gather_candidates(S, rank, sc);   // (2) block 0 holds every block's candidates; the peers are done
+    if (rank != 0) return;
+    rare = sc.sh_cnt > (uint32_t)kMaxCand;
+  } else {
+    reinterpret_cast<SubMax<T>*>(sc.cand)[tid] = sub;
   }
-  if (rank == 0)
-    for (int b = tid; b < kBins; b += kThreads) sc.bin_cur[b] = 0u;   // (the histogram is done with: it becomes the counting sort's)
-  cluster.sync();   // (2) block 0 holds every block's candidates; the peers are done
-  if (rank != 0) return;
-  const uint32_t n_pass = sc.sh_cnt;
-  if (n_pass > (uint32_t)kMaxCand) {   // many equal logits around the K-th place: the general way
-    radix_path<T>(row, vocab, K, row_idx, out_ids, out_probs, sc);
-    return;
-  }
-  float sum = 0.f;   // in rank order: the result does not depend on timing
-  for (int r = 0; r < S; ++r) sum += sc.x_sum[r] * exp2f_fast((value_of_key(sc.x_hi[r]) - row_max_f) * kLog2e);
-  unsigned long long* src = S == 1 ? sc.cand : sc.pool;
-  unsigned long long* dst = S == 1 ? sc.pool : sc.cand;
-  const uint32_t hi16 = top >> 16;
-  auto write_out = [&](unsigned long long c, uint32_t pos) {
-    out_ids[row_idx * K + pos] = (int32_t)(0xFFFFFFFFu - (uint32_t)c);
-    out_probs[row_idx * K + pos] = expf(value_of_key((uint32_t)(c >> 32)) - row_max_f) / sum;
-  };
-
-  // ---- counting sort: bin b holds the candidates whose upper key bits are hi16 - b (descending logit); those
-  // beyond the bins share the last one.  Inside a bin the larger 64-bit value (larger key, then smaller token id) goes first.
-  uint32_t big = 0u;
-  for (uint32_t i = tid; i < n_pass; i += kThreads)
-    big |= atomicAdd(&sc.bin_cur[min(hi16 - (uint32_t)(src[i] >> 48), (uint32_t)kBins - 1u)], 1u) >= kMaxBin ? 1u : 0u;
-  if (!__syncthreads_or((int)big)) {
-    {   // exclusive scan over the bins: four bins per thread, warp scans, then the warps' totals
-      const uint4 c = *reinterpret_cast<const uint4*>(&sc.bin_cur[4 * tid]);
-      static_assert(kBins == 4 * kThreads, "four bins per thread");
-      const uint32_t tot = c.x + c.y + c.z + c.w;
-      uint32_t incl = tot;
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += up;
-      }
-      if (lane == 31) sc.scan[warp] = incl;
-      __syncthreads();
-      uint32_t warp_base = lane < warp ? sc.scan[lane % kWarps] : 0u;
-      warp_base = __reduce_add_sync(0xFFFFFFFFu, warp_base);
-      const uint32_t ex = warp_base + incl - tot;
-      const uint4 st = make_uint4(ex, ex + c.x, ex + c.x + c.y, ex + c.x + c.y + c.z);
-      *reinterpret_cast<uint4*>(&sc.bin_start[4 * tid]) = st;
-      *reinterpret_cast<uint4*>(&sc.bin_cur[4 * tid]) = st;
-    }
-    __syncthreads();
-    for (uint32_t i = tid; i < n_pass; i += kThreads) {
-      const unsigned long long c = src[i];
-      dst[atomicAdd(&sc.bin_cur[min(hi16 - (uint32_t)(c >> 48), (uint32_t)kBins - 1u)], 1u)] = c;   // grouped by bin, any order inside
-    }
-    __syncthreads();
-    for (uint32_t i = tid; i < n_pass; i += kThreads) {
-      const unsigned long long mine = dst[i];
-      const uint32_t bin = min(hi16 - (uint32_t)(mine >> 48), (uint32_t)kBins - 1u);
-      const uint32_t first = sc.bin_start[bin], end = sc.bin_cur[bin];
-      if (first >= (uint32_t)K) continue;
-      uint32_t pos = first;
-      for (uint32_t j = first; j < end; ++j) pos += dst[j] > mine ? 1u : 0u;
-      if (pos < (uint32_t)K) write_out(mine, pos);
-    }
-    return;
-  }
-  // ---- a bin with very many candidates (equal logits, or logits far below the maximum): sort them all
-  int n_sort = 1;
-  while (n_sort < (int)n_pass) n_sort <<= 1;
-  for (int i = (int)n_pass + tid; i < n_sort; i += kThreads) src[i] = 0ull;   // padding sorts to the end
-  __syncthreads();
-  sort_descending(src, n_sort);
-  for (int i = tid; i < K; i += kThreads) write_out(src[i], (uint32_t)i);
+  if (rare) rare_row<T>(args, tau);
+  else finish_row<T, false>(args, tau, top, sc);
 }
 
 template <typename T, int NG>
-cudaError_t launch_next_dist(const T* logits, int64_t row_stride, int vocab, int K, int S, int subsets, int n_rows, int32_t* out_ids, float* out_probs,
-                             bool& configured, cudaStream_t s) {
+cudaError_t launch_next_dist(const NdArgs<T>& args, int S, int n_rows, bool& configured, cudaStream_t s) {
   auto kern = next_dist_kernel<T, NG>;
   if (!configured) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(NdScratch));
@@ -700,7 +907,7 @@ cudaError_t launch_next_dist(const T* logits, int64_t row_stride, int vocab, int
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kern, logits, row_stride, vocab, K, subsets, out_ids, out_probs);
+  return cudaLaunchKernelEx(&cfg, kern, args);
 }
 
 template <typename T>
@@ -717,12 +924,12 @@ int next_dist(pie_ctx* ctx, const void* logits, int n_rows, int vocab, int64_t r
     int subsets = 1;
     const int busy = std::min(kThreads, std::max(1, (n_groups + S - 1) / S));
     while (subsets < Elem<T>::VEC && busy * subsets * 2 < 3 * ((K + S - 1) / S)) subsets *= 2;
-    const T* p = static_cast<const T*>(logits);
+    const NdArgs<T> args = {static_cast<const T*>(logits), row_stride, vocab, K, subsets, out_ids, out_probs};
     bool* configured = ctx->nd_configured + (sizeof(T) == 2 ? 0 : 3);
     cudaError_t e;
-    if (NG == 2) e = launch_next_dist<T, 2>(p, row_stride, vocab, K, S, subsets, n_rows, out_ids, out_probs, configured[0], s);
-    else if (NG == 4) e = launch_next_dist<T, 4>(p, row_stride, vocab, K, S, subsets, n_rows, out_ids, out_probs, configured[1], s);
-    else e = launch_next_dist<T, 8>(p, row_stride, vocab, K, S, subsets, n_rows, out_ids, out_probs, configured[2], s);
+    if (NG == 2) e = launch_next_dist<T, 2>(args, S, n_rows, configured[0], s);
+    else if (NG == 4) e = launch_next_dist<T, 4>(args, S, n_rows, configured[1], s);
+    else e = launch_next_dist<T, 8>(args, S, n_rows, configured[2], s);
     if (e == cudaSuccess) return PIE_OK;
     // (a device that cannot place such clusters - fewer SMs per GPC, a partitioned GPU - refuses the launch: one block per row then)
     cudaGetLastError();

@@ -36,3 +36,75 @@ def test_ties_of_negative_logits_at_the_last_place(dtype, fill):
     z = torch.full((2, 30000), fill)
     z[:, 5:400] = torch.randn(2, 395, generator=torch.Generator().manual_seed(6)).abs()    # fewer entries above `fill` than K
     _check(z.to(dtype).cuda(), 600)
+
+
+def _placed(kind, n, V, seed):
+    """Rows whose K-th largest logit lies far below the largest: other sign, log-probabilities with a confident top, a common
+    offset that leaves fp32 little resolution, most of the vocabulary masked out (in one run, or all but every 37th token),
+    and all of it."""
+    g = torch.Generator().manual_seed(seed)
+    x = torch.randn(n, V, generator=g) * 2.5
+    if kind == "negative":
+        x = x - 8
+        x[:, 3] = 1.5
+    elif kind == "confident":
+        x[:, V // 2] += 40
+        x = torch.log_softmax(x, -1)
+    elif kind == "offset":
+        x = x + 1000
+    elif kind == "far offset":
+        x = x + 1e6
+    elif kind == "half masked":
+        x[:, V // 2:] = float("-inf")
+    elif kind == "few allowed":
+        x[:, V // 90 + 1:] = float("-inf")
+    elif kind == "every 37th":
+        keep = torch.arange(V) % 37 == 5
+        keep[1] = True
+        x[:, ~keep] = float("-inf")
+    elif kind == "lowest":
+        x[:, V // 2:] = torch.finfo(torch.float32).min
+        x[:, 9:V // 2] = float("-inf")
+    return x
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("kind", ["negative", "confident", "offset", "far offset", "half masked", "few allowed", "every 37th", "lowest"])
+def test_thresholds_beyond_the_histogram(kind, dtype):
+    from tests.test_gpu_next_dist import _check
+    for n, V, K in ((1, 40003, 256), (3, 9001, 1000), (40, 17000, 50), (160, 8000, 256), (2, 700, 256), (1, 70001, 1024)):
+        _check(_placed(kind, n, V, seed=V).to(dtype).cuda(), K)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("n,V", [(64, 128256), (1, 128256), (512, 8000)])
+def test_time_does_not_depend_on_where_the_logits_lie(n, V, dtype):
+    """A common offset or a confident top costs at most a second threshold (about 10 us), not the row again on one block: 4 - 27
+    times the time of centred logits while such rows were left to the radix selection, 1.0 - 2.1 times since."""
+    import paper_2510_24051_b200 as pie
+    from tests.test_gpu_next_dist import _ctx
+    ids = torch.empty(n, 256, dtype=torch.int32, device="cuda")
+    probs = torch.empty(n, 256, dtype=torch.float32, device="cuda")
+    ctx = _ctx()
+
+    def us(x):
+        for _ in range(3):
+            pie.pie_get_next_dist(ctx, x, 256, ids, probs)
+        best = 1e9
+        for _ in range(5):
+            torch.cuda.synchronize()
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(20):
+                pie.pie_get_next_dist(ctx, x, 256, ids, probs)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b) * 50)
+        return best
+    try:
+        centred = us(_placed("", n, V, 1).to(dtype).cuda())
+        for kind in ("negative", "confident"):
+            assert us(_placed(kind, n, V, 1).to(dtype).cuda()) <= 2.5 * centred + 2, kind
+    finally:
+        torch.cuda.synchronize()
+        pie.pie_destroy(ctx)
