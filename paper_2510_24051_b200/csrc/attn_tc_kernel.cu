@@ -155,11 +155,17 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
 }
 // 2^y for a pair on the FMA pipe: y = n + r with r in [-0.5, 0.5] (n by adding and subtracting 1.5 * 2^23), 2^r as the
 // polynomial of degree 5 with the smallest largest relative error there (Remez exchange in fp64; 1.8 * 2^-23 with its fp32
-// rounding, ex2.approx has 2 * 2^-23), n added to the exponent.  y is clamped to [-126, 126].
+// rounding, ex2.approx has 2 * 2^-23), n added to the exponent.  y is clamped to [-126, 126] except where it is NaN: the
+// operations leave the NaN 0x7FFFFFFF there, and with its low bits added to its exponent 0x7F7FFFFF, the largest number there is -
+// no sum the caller accepts, so that the chunk is done again with ex2.approx, which passes NaN on.
 __device__ __forceinline__ void exp2_poly(uint64_t y2, float& e0, float& e1) {
   float y0, y1;
   unpack_f32x2(y2, y0, y1);
-  y2 = pack_f32x2(fminf(fmaxf(y0, -126.f), 126.f), fminf(fmaxf(y1, -126.f), 126.f));
+  auto clamp = [](float y) {
+    asm("max.NaN.f32 %0, %0, %1;\n\tmin.NaN.f32 %0, %0, %2;" : "+f"(y) : "f"(-126.f), "f"(126.f));
+    return y;
+  };
+  y2 = pack_f32x2(clamp(y0), clamp(y1));
   const uint64_t z2 = add_f32x2(y2, pack_f32x2(12582912.f, 12582912.f));
   const uint64_t n2 = add_f32x2(z2, pack_f32x2(-12582912.f, -12582912.f));
   const uint64_t r2 = fma_f32x2(n2, pack_f32x2(-1.f, -1.f), y2);

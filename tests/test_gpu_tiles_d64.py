@@ -45,3 +45,23 @@ def test_masks_without_positions_in_a_half():
     masks[1][7, :] = False                       # an empty row
     masks[1][9, :190] = False
     _run([(48, 256), (40, 200)], 8, 2, 16, masks)
+
+
+@pytest.mark.parametrize("P", [8, 16, 32])
+def test_nan_key_shows_at_every_position(P):
+    """A NaN key that every row sees reaches every output of its kv head - no output of another - wherever it lies in a KV tile."""
+    from tests._util import SmallBatch, random_seqs
+    from tests.test_gpu_matrix import run_gpu
+    seqs = random_seqs(np.random.RandomState(P), [(64, 1024)], 8, 2, 64)
+    args = SmallBatch(seqs, 8).paged(P, order="random", seed=P)
+    lse = []
+    for pos in (0, 1, 2, 16, 17, 47, 64, 65, 80, 127, 256, 272, 959):
+        page, slot = args["page_indices"][pos // P], pos % P
+        pool = {p: (k.copy(), v.copy()) for p, (k, v) in args["pool"].items()}
+        pool[int(page)][0][slot, 0, 5] = np.nan
+        O, L, info = run_gpu(dict(args, pool=pool), max(pool) + 1, 2, 64, "bf16")
+        assert info["num_tile_items"] > 0
+        assert np.isnan(O[:, :4]).all(), pos
+        assert np.isfinite(O[:, 4:]).all() and np.isfinite(L[:, 4:]).all(), pos
+        lse.append(L[:, :4])
+    assert all(np.array_equal(x, lse[0], equal_nan=True) for x in lse)
