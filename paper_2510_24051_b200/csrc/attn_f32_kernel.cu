@@ -64,8 +64,60 @@ struct F32Cfg {
   static_assert(RW * TW * MR * OSTRIDE * 4 <= RING, "the partials of a block fit over its idle rings");
 };
 
+// The items of a block that had an output that is not finite, once more: a row must not feel the K and V of a position it does
+// not see, whatever they hold, and the tiles below multiply the V of such a position by a weight of zero - which an infinity or
+// NaN survives.  Here a warp takes a row at a time, straight from the pool, and passes over the positions that are hidden from
+// it.  (As the last thing the kernel does it costs about 1 % of a mixed
+// step, 88.1 -> 89.0 us; inside the item loop, even behind a branch never taken, 2 - 4 % of decode launches and up to 5 % of chunks.)
+template <int D>
+__device__ __noinline__ void careful_items(const AttnParams& p, const PoolGeom& g, float scale) {
+  for (int it = p.cta_ptr[blockIdx.x]; it < p.cta_ptr[blockIdx.x + 1]; ++it) {
+    const PieItem& item = p.items[it];
+    const int lane = threadIdx.x & 31;
+    for (int row = threadIdx.x >> 5; row < item.nrows; row += blockDim.x >> 5) {
+      const int gr = item.row0 + row, tok = gr / p.G, lim = item.kv_len - item.q_len + tok;
+      const int64_t oi = (int64_t)(item.q_start + tok) * p.n_q_heads + item.kv_head * p.G + gr % p.G;
+      const uint32_t* mrow = p.mask + item.mask_word_off + (int64_t)tok * item.mask_row_words;
+      float q[D / 32], acc[D / 32], m = kNegInf, l = 0.f;
+#pragma unroll
+      for (int k = 0; k < D / 32; ++k) {
+        q[k] = __ldg(reinterpret_cast<const float*>(p.q) + oi * D + k * 32 + lane);
+        acc[k] = 0.f;
+      }
+      for (int pg = item.page_begin; pg < item.page_end; ++pg) {
+        const int2 kept = __ldg(&p.kept[pg]);
+        const uint8_t* page = reinterpret_cast<const uint8_t*>(p.pool) + (int64_t)kept.x * p.page_bytes + (int64_t)item.kv_head * 2 * g.block_bytes + (lane & 3) * 4;
+        const int pos0 = (int)((uint32_t)kept.y & ~PIE_KEPT_NEEDS_MASK) * g.page_size;
+        for (int slot = 0; slot < g.page_size; ++slot) {
+          const int pos = pos0 + slot;
+          if (pos >= item.kv_len) break;
+          if (((uint32_t)kept.y & PIE_KEPT_NEEDS_MASK) && !(item.mask_row_words ? (__ldg(mrow + (pos >> 5)) >> (pos & 31)) & 1u : pos <= lim)) continue;
+          float x = 0.f;
+#pragma unroll
+          for (int k = 0; k < D / 32; ++k) x += q[k] * *reinterpret_cast<const float*>(page + pie_chunk_offset(g.slab_bytes, slot, k * 8 + (lane >> 2)));
+          for (int sft = 16; sft > 0; sft >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, sft);
+          x *= scale;
+          const float m_new = fmaxf(m, x), m_use = m_new == kNegInf ? 0.f : m_new, alpha = expf(m - m_use), e = expf(x - m_use);
+          m = m_new;
+          l = l * alpha + e;
+#pragma unroll
+          for (int k = 0; k < D / 32; ++k)
+            acc[k] = acc[k] * alpha + e * *reinterpret_cast<const float*>(page + g.block_bytes + pie_chunk_offset(g.slab_bytes, slot, k * 8 + (lane >> 2)));
+        }
+      }
+      const float inv = l > 0.f ? 1.f / l : 0.f, lse = l > 0.f ? m + logf(l) : kNegInf;
+      const int64_t si = (int64_t)item.partial_slot * p.slot_rows + row;
+      const bool last = item.partial_slot < 0;
+      float* o = last ? reinterpret_cast<float*>(p.out) + oi * D : p.ws_o + si * D;
+#pragma unroll
+      for (int k = 0; k < D / 32; ++k) o[k * 32 + lane] = acc[k] * inv;
+      if (lane == 0) (last ? p.lse[oi] : p.ws_lse[si]) = lse;
+    }
+  }
+}
+
 template <int D, int MR, int RW, int TW, int TOK>
-__global__ void __launch_bounds__(RW * TW * 32, RW > 1 && D == 64 ? 2 : 1) attn_f32_kernel(const AttnParams p, const PoolGeom g, const float scale, const int page_shift) {
+__global__ void __launch_bounds__(RW * TW * 32, RW > 1 && D == 64 ? 2 : 1) attn_f32_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ PoolGeom g, const float scale, const int page_shift) {
   using C = F32Cfg<D, MR, RW, TW, TOK>;
   constexpr int RT = MR / 4;        // rows per lane
   constexpr int NC = D / 32;        // 16-byte output columns per lane
@@ -98,6 +150,7 @@ __global__ void __launch_bounds__(RW * TW * 32, RW > 1 && D == 64 ? 2 : 1) attn_
     tok_off[j] = (t >> page_shift) * vp + (t & (P - 1)) * 128;
   }
   uint32_t cnt = 0;   // tiles of this token group so far (ring position)
+  int odd_items = 0;  // an item had an output that is not finite
   const int it0 = p.cta_ptr[blockIdx.x], it1 = p.cta_ptr[blockIdx.x + 1];
   for (int it = it0; it < it1; ++it) {
     const PieItem item = p.items[it];
@@ -315,6 +368,7 @@ __global__ void __launch_bounds__(RW * TW * 32, RW > 1 && D == 64 ? 2 : 1) attn_
       if (tg == 0) dst[D] = m_run[i], dst[D + 1] = l_run[i];
     }
     __syncthreads();
+    bool odd = false;
     for (int x = threadIdx.x; x < item.nrows * (D / 4); x += C::THREADS) {
       const int row = x / (D / 4), ch = x % (D / 4), gr = item.row0 + row;
       const float* src = part + row * C::OSTRIDE;
@@ -334,6 +388,7 @@ __global__ void __launch_bounds__(RW * TW * 32, RW > 1 && D == 64 ? 2 : 1) attn_
       const float inv = L > 0.f ? 1.f / L : 0.f;
       const float lse = L > 0.f ? M + logf(L) : kNegInf;
       a.x *= inv, a.y *= inv, a.z *= inv, a.w *= inv;
+      odd |= !(fabsf(a.x) + fabsf(a.y) + fabsf(a.z) + fabsf(a.w) < __builtin_huge_valf());   // (a sum that overflows only costs the second time)
       if (item.partial_slot < 0) {
         const int64_t oi = (int64_t)(item.q_start + gr / p.G) * p.n_q_heads + item.kv_head * p.G + gr % p.G;
         *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + oi * D + ch * 4) = a;
@@ -345,8 +400,9 @@ __global__ void __launch_bounds__(RW * TW * 32, RW > 1 && D == 64 ? 2 : 1) attn_
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the partials were written where the next item's copies land
-    __syncthreads();
+    odd_items |= __syncthreads_or(odd);
   }
+  if (odd_items) careful_items<D>(p, g, scale);   // (behind a block barrier: their results so far are written over)
   if (p.late_trigger) pie_pdl_launch_dependents();
 }
 

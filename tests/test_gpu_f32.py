@@ -46,3 +46,31 @@ def test_fp32_unit_cut_across_blocks():
         O, L, info = run_gpu(gpu_args, max(args["pool"]) + 1, 2, 64, "f32")
         assert info["num_merge_groups"] > 0
         assert np.abs(O - O_ref).max() <= TOL and np.abs(L - L_ref).max() <= TOL
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("D,P", [(64, 8), (64, 16), (64, 32), (128, 16), (128, 32)])
+def test_fp32_hidden_rows_may_hold_anything(D, P, bad):
+    """K and V of a position that a row does not see do not reach it, even where they are infinite or NaN: a later token of
+    the row's own chunk, a position hidden by an explicit mask.  Rows that see it show it."""
+    import paper_2510_24051_b200 as pie
+    from tests._util import SmallBatch, oracle_on, random_seqs
+    from tests.test_gpu_matrix import run_gpu
+    rng = np.random.RandomState(P)
+    seqs = random_seqs(rng, [(40, 70), (4, 90), (2, 33)], 4, 1, D)
+    seqs[1]["mask"] = rng.rand(4, 90) < 0.7
+    seqs[1]["mask"][:, 50] = [False, True, False, False]
+    hidden = [(0, 55), (1, 50), (2, 32)]                 # (request, position): the chunk's 26th token, masked for three rows of four, the last token
+    clean = oracle_on(SmallBatch(seqs, 4).paged(P, order="random", seed=5))
+    for r, j in hidden:
+        seqs[r]["K"][j, 0, 3] = np.nan
+        seqs[r]["V"][j] = bad
+    args = SmallBatch(seqs, 4).paged(P, order="random", seed=5)
+    sees = np.zeros(46, dtype=bool)
+    sees[25:40] = sees[41] = sees[45] = True
+    for flags in (0, pie.PIE_PLAN_FORCE_SIMPLE):
+        gpu_args = dict(args, pool={p: (k.copy(), v.copy()) for p, (k, v) in args["pool"].items()})
+        O, L, info = run_gpu(gpu_args, max(args["pool"]) + 1, 1, D, "f32", flags)
+        assert (info["num_simple_rows"] == 0) == (flags == 0)
+        assert np.abs(O[~sees] - clean[0][~sees]).max() <= TOL and np.abs(L[~sees] - clean[1][~sees]).max() <= TOL
+        assert np.isnan(O[sees]).all()
