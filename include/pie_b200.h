@@ -210,7 +210,8 @@ typedef struct pie_plan_info {
  * vertical-batching rule of Section 5.2; reading rows an EARLIER request appends is legal,
  * because the whole batch is appended before any request attends),
  * PIE_ERR_BATCH_TOO_LARGE, PIE_ERR_MASK.  *out is set only on success.  The upload is enqueued on
- * `stream` from memory of the library's own; forwards on any stream are ordered behind it. */
+ * `stream` from memory of the library's own; forwards on any stream are ordered behind it.  A stream that is
+ * being captured is refused with PIE_ERR_CUDA (the capture stays valid): plan first, capture the forward. */
 int pie_plan_forward(pie_ctx* ctx, const pie_batch_desc* batch, void* stream, pie_plan** out);
 /* Ends the plan's life.  The context keeps a few destroyed plans - host arrays, pinned upload
  * image and device arrays - and pie_plan_forward reuses them, so a loop that plans every step

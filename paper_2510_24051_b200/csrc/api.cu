@@ -691,9 +691,17 @@ int pie_copy_kvpage(pie_ctx* ctx, int32_t n, const int32_t* src, const int32_t* 
 // of the one plan (small decode batches, plan + forward: 41 us a step when every plan waited for its upload).
 static const size_t kParkedPlans = 4;
 
+// Event queries and waits of this thread do not disturb a capture that goes on elsewhere while one of these lives.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // The plan's pinned image may be written again once its upload is over.
 static bool upload_over(const pie_plan* plan) {
   if (!plan->upload_pending) return true;
+  RelaxedCapture relaxed;
   const cudaError_t e = cudaEventQuery(plan->uploaded);
   if (e == cudaSuccess) plan->upload_pending = false;
   else cudaGetLastError();   // (not ready)
@@ -701,6 +709,7 @@ static bool upload_over(const pie_plan* plan) {
 }
 static cudaError_t wait_uploaded(const pie_plan* plan) {
   if (!plan->upload_pending) return cudaSuccess;
+  RelaxedCapture relaxed;
   const cudaError_t e = cudaEventSynchronize(plan->uploaded);
   if (e == cudaSuccess) plan->upload_pending = false;
   return e;
@@ -717,11 +726,7 @@ static int order_behind_upload(pie_ctx* ctx, const pie_plan* plan, cudaStream_t 
   if (cap != cudaStreamCaptureStatusNone) {
     // the graph may be replayed on any stream, at any time: the upload has to be over, and the capture must not
     // see the wait
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    PIE_CUDA(ctx, cudaThreadExchangeStreamCaptureMode(&mode));
-    const cudaError_t e = wait_uploaded(plan);
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    PIE_CUDA(ctx, e);
+    PIE_CUDA(ctx, wait_uploaded(plan));
     return PIE_OK;
   }
   if (plan->used && upload_over(plan)) return PIE_OK;
@@ -775,7 +780,17 @@ int pie_plan_forward(pie_ctx* ctx, const pie_batch_desc* batch, void* stream, pi
     cudaStream_t s = (cudaStream_t)stream;
     const PlanLayout L = pie_plan_layout(ctx, plan);
     cudaError_t e = cudaSetDevice(ctx->cfg.device);
-    if (e == cudaSuccess) e = wait_uploaded(plan);
+    // A captured upload would run with every replay, from a pinned image and into device arrays that serve other plans by then.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (e == cudaSuccess) e = cudaStreamIsCapturing(s, &cap);
+    if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+      ctx->cuda_error = std::string("plan upload: ") + (e != cudaSuccess ? cudaGetErrorString(e) : "the stream is being captured");
+      cudaGetLastError();
+      pie_plan_release_scratch(plan);
+      give_back();
+      return PIE_ERR_CUDA;
+    }
+    e = wait_uploaded(plan);
     if (e == cudaSuccess && plan->idle_pending) {   // the upload goes behind the forward that last read the device arrays
       e = cudaStreamWaitEvent(s, plan->idle, 0);
       plan->idle_pending = false;

@@ -65,3 +65,50 @@ def test_plans_in_flight_on_one_and_on_two_streams():
         del g
         pie.pie_plan_destroy(plan)
         assert pie.pie_get_last_device_status(gp.ctx) == 0
+
+
+def test_planning_while_a_stream_is_captured():
+    """On the captured stream planning is refused and leaves the capture as it was - the upload must not become part of the
+    graph, whose replays would read a pinned image that serves other plans by then.  Next to a capture of another stream a plan
+    is made and run as ever."""
+    import paper_2510_24051_b200 as pie
+    from tests._gpu import GpuPool
+    wl, steps = _loop_batches(6)
+    with GpuPool(wl.num_pages, wl.P, wl.H_q, wl.H_kv, wl.D, wl.dtype) as gp:
+        gp.install(wl)
+        q, k, v = wl.q("cuda"), wl.k_new("cuda"), wl.v_new("cuda")
+        args = [{n: b[n] for n in ("qo_indptr", "page_indptr", "page_indices", "last_page_len")} for b in steps]
+        ref, out = [(torch.zeros_like(q), torch.zeros(wl.T, wl.H_q, device="cuda")) for _ in range(2)]
+        for _ in range(2):                                # (the second time with a parked plan: nothing is allocated any more)
+            plan = pie.pie_plan_forward(gp.ctx, **args[3])
+            pie.pie_forward(gp.ctx, plan, q, k, v, *ref)
+            torch.cuda.synchronize()
+            pie.pie_plan_destroy(plan)
+        free0 = pie.pie_num_free_kvpages(gp.ctx)
+        x, y = torch.ones(64, device="cuda"), torch.zeros(64, device="cuda")
+        s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+        busy = torch.zeros(1 << 26, device="cuda")
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s1):
+            with pytest.raises(pie.PieError) as e:
+                pie.pie_plan_forward(gp.ctx, **args[3])
+            assert e.value.status == pie.PIE_ERR_CUDA
+            with torch.cuda.stream(s2):
+                for _ in range(20):
+                    busy.add_(1.0)                    # the upload queues behind this
+                plan = pie.pie_plan_forward(gp.ctx, **args[3])
+                pie.pie_forward(gp.ctx, plan, q, k, v, *out)
+                pie.pie_forward(gp.ctx, plan, q, k, v, *out)
+                pie.pie_plan_destroy(plan)
+            torch.add(x, 1.0, out=y)
+        g.replay()
+        torch.cuda.synchronize()
+        assert (y == 2).all() and torch.equal(out[0], ref[0]) and torch.equal(out[1], ref[1])
+        assert pie.pie_num_free_kvpages(gp.ctx) == free0
+        for a in args:                                    # (and planning goes on)
+            plan = pie.pie_plan_forward(gp.ctx, **a)
+            pie.pie_forward(gp.ctx, plan, q, k, v, *out)
+            pie.pie_plan_destroy(plan)
+        torch.cuda.synchronize()
+        assert pie.pie_get_last_device_status(gp.ctx) == 0
