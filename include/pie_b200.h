@@ -303,8 +303,10 @@ int pie_debug_bounded_wait(pie_ctx* ctx, void* stream);
  *     are handed back when the call returns and rejoin the free list once the work enqueued on
  *     `stream` has finished (one CUDA event per such call, recycled - a host-side object, no device
  *     memory).
- *   - A batch whose plan arrays plus split partials need more than PIE_STATIC_SCRATCH_BYTES is
- *     refused with PIE_ERR_BATCH_TOO_LARGE and nothing is enqueued.
+ *   - A batch whose plan arrays plus split partials need more than PIE_STATIC_SCRATCH_BYTES is laid out
+ *     again with as few partials as its requests allow (whole row-tile units, no unit-per-block decode lists;
+ *     results then differ from pie_forward's by rounding).  If that does not fit either it is refused with
+ *     PIE_ERR_BATCH_TOO_LARGE and nothing is enqueued.
  *   - The first call on a device looks up the array's device address (one cudaGetSymbolAddress,
  *     with that device current); make that first call before any stream capture.
  *   - All calls share the one array, which keeps the previous call's contents.  Nothing in it has

@@ -1593,7 +1593,13 @@ extern "C" int pie_forward_static_scratch(pie_ctx* ctx, const pie_batch_desc* ba
   plan.ctx = ctx;
   const int saved_overlap = ctx->options[PIE_OPT_OVERLAP];
   ctx->options[PIE_OPT_OVERLAP] = 2;  // this entry point enqueues its kernels one after the other
-  int rc = pie_build_plan(ctx, batch, &plan);
+  // A plan that spends partials on speed may not fit the scratch: then the batch is laid out again with less of them.
+  int rc;
+  for (;; ++ctx->lean) {
+    rc = pie_build_plan(ctx, batch, &plan);
+    if (rc != PIE_OK || ctx->lean == 2 || pie_plan_layout(ctx, &plan).total <= (size_t)PIE_STATIC_SCRATCH_BYTES) break;
+  }
+  ctx->lean = 0;
   ctx->options[PIE_OPT_OVERLAP] = saved_overlap;
   if (rc != PIE_OK) return rc;   // (a failed build has given its borrowed pages back)
   // Pages borrowed for requests without output KvPages: on every way out from here they are handed to

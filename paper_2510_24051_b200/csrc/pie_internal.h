@@ -221,6 +221,10 @@ struct pie_ctx {
   int max_clusters[2][3] = {{-1, -1, -1}, {-1, -1, -1}};   // pie_split_max_clusters: of 2 / 4 / 8 blocks; -1: not asked yet
   bool f32_configured[3] = {false, false, false};   // (items of <= 4, <= 16, 64 rows)
   bool tc_configured = false, split_configured = false, split_pair_configured = false, tile_configured = false, nd_configured[6] = {false, false, false, false, false, false};   // kernel attributes set for this context's device
+  // How much scratch the next plan may take for speed (pie_forward_static_scratch): 0 as much as it likes; 1 no unit is cut
+  // that can stay whole, so that only cascades and shares over all warps write partials; 2 moreover no unit-per-block decode lists
+  // (fp32: row by row, without any list).
+  int lean = 0;
   // The block-local work list of the latest decode batch.  Consecutive steps of a serving loop bring the same
   // requests with the same page counts (a request grows by a page every page_size steps), and then the list is
   // the same up to the fields copied from the request records: the planner reuses it instead of dealing the

@@ -702,7 +702,7 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
 // Otherwise (false, the units stay as they are) shares over all warps of the chip, laid out in advance.
 static bool pick_cluster(pie_ctx* ctx, std::vector<Unit>& units, bool plain, int64_t W, int sms, int hp, bool side_by_side, bool long_launch,
                          int* blocks, int* warps) {
-  if (units.empty() || !plain || side_by_side || sms != ctx->n_sms || (ctx->options[PIE_OPT_NO_FUSION] & (2 | 8 | 16))) return false;
+  if (units.empty() || !plain || side_by_side || sms != ctx->n_sms || ctx->lean > 1 || (ctx->options[PIE_OPT_NO_FUSION] & (2 | 8 | 16))) return false;
   // (Long launches on 8-token pages stay with the chunk list, although blocks of their own are 1.5 - 6 % faster there as well:
   //  tests/test_gpu_full_configs.py holds them to chunks of odd page counts that merge in a launch of their own.)
   if (long_launch && ctx->cfg.page_size == 8) return false;
@@ -1206,7 +1206,7 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
   // (head groups above 16 - multi-query models - do not fit the split-KV kernel's 16 rows per warp: every request
   //  of such a context has more than 16 rows and runs on the row-tile kernel)
   const bool f32 = cfg.dtype == PIE_DTYPE_F32;   // fp32 pools: both launch lists run on the fp32 kernel (items of at most 16 / of 64 rows)
-  const bool tiles_ok = (f32 || pie_split_supported(ctx) || (pie_tc_supported(ctx) && G > 16)) && !(b->flags & PIE_PLAN_FORCE_SIMPLE);
+  const bool tiles_ok = (f32 || pie_split_supported(ctx) || (pie_tc_supported(ctx) && G > 16)) && !(b->flags & PIE_PLAN_FORCE_SIMPLE) && !(f32 && ctx->lean > 1);
   std::vector<Unit> split_units, tile_units;
   plan->simple_rows.clear();
   // (8-token pages: the mma.sync row-tile kernel behind PIE_PLAN_NO_TENSOR_TILES has no instantiation, the flag is ignored)
@@ -1409,9 +1409,10 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
   // row tiles first: the cascade pieces get their partial slots, which the split units of the
   // cascaded requests then name as further sources of their merge groups
   UnitSlots tile_slots;
+  const int lean_slack = 1 << 30;   // (no unevenness is worth a cut)
   // (fp32: a page of 16 tokens takes a block of 64 rows about 1 us, the merge launch 4 - 5 us)
-  if (f32) partition(tile_units, tile_sms * pie_f32_blocks_per_sm(ctx, true), 4, TILE_ROWS, true, plan->tile, &tile_slots, 5);
-  else if (!plan->tile_tc) partition(tile_units, tile_sms, 8, TILE_ROWS, true, plan->tile, &tile_slots);
+  if (f32) partition(tile_units, tile_sms * pie_f32_blocks_per_sm(ctx, true), 4, TILE_ROWS, true, plan->tile, &tile_slots, ctx->lean ? lean_slack : 5);
+  else if (!plan->tile_tc) partition(tile_units, tile_sms, 8, TILE_ROWS, true, plan->tile, &tile_slots, ctx->lean ? lean_slack : 200);
   else {
     // tcgen05 row tiles, in units of 16 tokens (about 0.2 us of a CTA; with 8-token pages 0.3): shares of at least 32, a
     // cut list costs 50 and 0.35 per piece.  Measured, us per step, 32 / 8 heads of 128, 16-token pages, whole against
@@ -1419,7 +1420,7 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
     // 4 x 128 behind 4,000 67 / 58, a prompt of 1,500 32 / 65; whole units on as many CTAs as there are units instead of one
     // per 512 tokens of the launch: a prompt of 64 tokens 25.6 -> 6.8, one of 300 30.9 -> 10.9 (64-wide heads, 32-token pages).
     const double k = P == 8 ? 0.7 : 1.0;
-    partition(tile_units, tile_sms, 512 / P, TILE_ROWS, true, plan->tile, &tile_slots, (int)(k * 50 * 16 / P), k * 0.35 * 16 / P);
+    partition(tile_units, tile_sms, 512 / P, TILE_ROWS, true, plan->tile, &tile_slots, ctx->lean ? lean_slack : (int)(k * 50 * 16 / P), k * 0.35 * 16 / P);
   }
   // merge groups of the larger cascaded requests (row-tile items over their private pages): add the slots of
   // the cascade pieces that hold the same rows
@@ -1479,7 +1480,7 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
     if (f32) {
       // one share per block; whole units while the fullest block stays within the merge launch of the average
       // (a block takes a 16-token page in about 0.1 us, the launch 4 - 5 us)
-      partition(split_units, split_sms * pie_f32_blocks_per_sm(ctx, false), 16, max_rows, true, plan->split, nullptr, 45);
+      partition(split_units, split_sms * pie_f32_blocks_per_sm(ctx, false), 16, max_rows, true, plan->split, nullptr, ctx->lean ? lean_slack : 45);
       plan->split.n_static = (int32_t)plan->split.items.size();
     } else if (int c_blocks = 0, c_warps = 0; pick_cluster(ctx, split_units, plain_units, W, split_sms, hp, plan->overlap, long_launch, &c_blocks, &c_warps)) {
       partition_cluster(split_units, c_blocks, c_warps, P == 8 ? 2 : 1, max_rows, plan->split);
