@@ -252,7 +252,7 @@ PlanLayout pie_plan_layout(const pie_ctx* ctx, const pie_plan* plan) {
   L.upload = off;
   const size_t D = ctx->cfg.head_dim;
   for (int k = 0; k < 2; ++k) {
-    const size_t n_slots = lls[k]->cluster > 0 ? 0 : (size_t)lls[k]->n_slots;   // (clusters merge in shared memory)
+    const size_t n_slots = (size_t)lls[k]->partial_slots();
     L.ws_o[k] = place(n_slots * lls[k]->slot_rows * D * 4);
     L.ws_lse[k] = place(n_slots * lls[k]->slot_rows * 4);
   }

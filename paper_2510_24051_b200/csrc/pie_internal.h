@@ -116,6 +116,7 @@ struct PieLaunchList {           // one tile-kernel launch (split-KV decode, or 
   bool grid_merge = false;       // split-KV: cut units are merged inside the kernel by their last piece (one counter per slot behind d_work_ctr)
   int32_t cluster = 0;           // split-KV: blocks of the cluster that owns a unit (decode_cluster_kernel); 0: attn_split_kernel
   int32_t cluster_warps = 0;     // ... and warps of each of these blocks
+  int32_t partial_slots() const { return cluster > 0 ? 0 : n_slots; }   // slots with fp32 partials in device memory (clusters merge in shared memory)
   int32_t heads_per_unit = 1;    // split-KV: 2 = every item covers kv heads 2 kv_head and 2 kv_head + 1 (rows of the first, then of the second)
   // device copies
   PieItem* d_items = nullptr;

@@ -1650,8 +1650,8 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
   info.num_merge_groups = (int32_t)(plan->split.merges.size() + plan->tile.merges.size());
   info.kept_pages = (int64_t)plan->kept.size() / 2;
   info.mask_words = (int64_t)plan->mask_words.size();
-  info.workspace_bytes = ((int64_t)plan->split.n_slots * plan->split.slot_rows +
-                          (int64_t)plan->tile.n_slots * plan->tile.slot_rows) * (cfg.head_dim + 1) * 4;
+  info.workspace_bytes = ((int64_t)plan->split.partial_slots() * plan->split.slot_rows +
+                          (int64_t)plan->tile.partial_slots() * plan->tile.slot_rows) * (cfg.head_dim + 1) * 4;
   info.side_by_side_sms = plan->overlap ? std::min(plan->tile.grid, ctx->n_sms) : 0;
   info.split_unit_kv_heads = plan->split.items.empty() ? 1 : plan->split.heads_per_unit;
   info.reserved0 = 0;

@@ -718,3 +718,23 @@ def test_worker_threads_come_and_go_with_their_context():
             pie.pie_destroy(c)
     assert np.array_equal(image(keep, wl, (mi, mb)), want)
     pie.pie_destroy(keep)
+
+
+def test_workspace_bytes_are_those_of_partials_in_device_memory():
+    """Decode units that own a block or a cluster of blocks merge in shared memory: no device scratch.  With shares over all warps
+    (PIE_OPT_NO_FUSION bit 4) pieces leave fp32 partials, and row tiles that are cut do."""
+    for bits, scratch in ((0, False), (16, True)):
+        ctx = pie.pie_create(4096, 16, 32, 8, 128, "bf16", 64, 4096, device=-1)
+        try:
+            pie.pie_set_option(ctx, pie.PIE_OPT_NO_FUSION, bits)
+            ids = pie.pie_alloc_kvpages(ctx, 1200)
+            plan = pie.pie_plan_forward(ctx, [0, 1, 2, 3], [0, 400, 500, 1000], ids[:1000], [16, 3, 9])
+            info = pie.pie_plan_get_info(plan)
+            assert info["num_split_items"] > 24 and (info["workspace_bytes"] > 0) == scratch
+            pie.pie_plan_destroy(plan)
+            plan = pie.pie_plan_forward(ctx, [0, 64], [0, 400], ids[:400], [16])       # one short chunk behind a long prefix
+            info = pie.pie_plan_get_info(plan)
+            assert info["num_merge_groups"] > 0 and info["workspace_bytes"] == info["num_tile_items"] * 256 * 129 * 4
+            pie.pie_plan_destroy(plan)
+        finally:
+            pie.pie_destroy(ctx)

@@ -27,6 +27,7 @@ def test_static_scratch_forward_matches_planned_forward(name):
     with GpuPool(wl.num_pages, wl.P, wl.H_q, wl.H_kv, wl.D, wl.dtype) as gp:
         gp.install(wl)
         pie.pie_set_option(gp.ctx, pie.PIE_OPT_OVERLAP, 2)      # the static-scratch call never runs kernels side by side
+        pie.pie_set_option(gp.ctx, pie.PIE_OPT_NO_FUSION, 16)   # (units in clusters of blocks merge in shared memory: no partials)
         q, k, v = wl.q("cuda"), wl.k_new("cuda"), wl.v_new("cuda")
         plan = gp.plan(wl)
         assert pie.pie_plan_get_info(plan)["workspace_bytes"] > 0       # the scratch partials are in use (merged in the kernel or by the merge launch)
@@ -42,6 +43,34 @@ def test_static_scratch_forward_matches_planned_forward(name):
             assert pie.pie_get_last_device_status(gp.ctx) == 0
             assert torch.equal(out, ref_out), f"call {call}"
             assert torch.equal(lse, ref_lse), f"call {call}"
+        check_close(out.double().cpu().numpy(), lse.double().cpu().numpy(), O_ref, L_ref, wl.dtype, wl.qo_indptr)
+
+
+@pytest.mark.parametrize("name", ["batched_decode", "long_context_policy", "mixed_prefill_decode", "four_long_decodes"])
+def test_static_scratch_forward_as_plans_are_by_default(name):
+    """The same with the lists the planner makes by default: a block or a cluster of blocks per decode unit, no partial in the
+    scratch."""
+    import paper_2510_24051_b200 as pie
+    from tests._gpu import GpuPool, check_close
+    from tests._util import run_oracle
+    from workloads import configs
+    wl = configs.batched_decode(R=4, num_pages=4096) if name == "four_long_decodes" else configs.small(name)
+    O_ref, L_ref, _ = run_oracle(wl)
+    with GpuPool(wl.num_pages, wl.P, wl.H_q, wl.H_kv, wl.D, wl.dtype) as gp:
+        gp.install(wl)
+        pie.pie_set_option(gp.ctx, pie.PIE_OPT_OVERLAP, 2)
+        q, k, v = wl.q("cuda"), wl.k_new("cuda"), wl.v_new("cuda")
+        plan = gp.plan(wl)
+        info = pie.pie_plan_get_info(plan)
+        assert info["num_split_items"] > 0 and (info["workspace_bytes"] == 0 or info["num_tile_items"] > 0)
+        ref_out, ref_lse = gp.forward(plan, q, k, v)
+        pie.pie_plan_destroy(plan)
+        mi, mb = wl.mask_bytes()
+        out, lse = torch.full_like(ref_out, float("nan")), torch.full_like(ref_lse, float("nan"))
+        pie.pie_forward_static_scratch(gp.ctx, wl.qo_indptr, wl.page_indptr, wl.page_indices, wl.last_page_len, q, k, v, out, lse, mi, mb)
+        torch.cuda.synchronize()
+        assert pie.pie_get_last_device_status(gp.ctx) == 0
+        assert torch.equal(out, ref_out) and torch.equal(lse, ref_lse)
         check_close(out.double().cpu().numpy(), lse.double().cpu().numpy(), O_ref, L_ref, wl.dtype, wl.qo_indptr)
 
 
