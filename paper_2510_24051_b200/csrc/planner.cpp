@@ -359,6 +359,44 @@ contiguous:
   ll.cta_ptr.push_back((int32_t)ll.items.size());
 }
 
+// Whole units for many thousands of them: the largest first, dealt to the CTAs there and back.  Their sum evens out without
+// looking for the least loaded CTA every time, which takes 0.1 us a unit: 4,096 fp32 requests of up to 100 tokens, 32 heads of 64,
+// 15.4 -> 10.3 ms of planning and upload for a forward of 1.8.  (Contiguous equal shares are as cheap, but their forwards took 7 - 21 % longer.)
+// False where a CTA gets fewer than a dozen units or one of them is large against its share.
+bool deal_in_turns(const std::vector<Unit>& units, int grid, int slot_rows, PieLaunchList& ll) {
+  const int64_t n = (int64_t)units.size();
+  int64_t W = 0;
+  int max_unit = 0;
+  for (const Unit& u : units) {
+    W += u.page_end - u.page_begin;
+    max_unit = std::max(max_unit, u.page_end - u.page_begin);
+  }
+  if (n < 12 * (int64_t)grid || max_unit * 8 > W / grid) return false;
+  ll.merges.clear();
+  ll.n_slots = 0;
+  ll.slot_rows = slot_rows;
+  ll.grid = grid;
+  ll.n_static = 0;
+  ll.cta_ptr.resize((size_t)grid + 1);
+  const int32_t each = (int32_t)(n / grid), rest = (int32_t)(n % grid), last_turn_back = each & 1;
+  ll.cta_ptr[0] = 0;
+  for (int c = 0; c < grid; ++c) ll.cta_ptr[c + 1] = ll.cta_ptr[c] + each + ((last_turn_back ? grid - 1 - c : c) < rest ? 1 : 0);
+  std::vector<int32_t> place((size_t)max_unit + 1, 0);   // of the next unit of a size, in descending order
+  for (const Unit& u : units) ++place[max_unit - (u.page_end - u.page_begin)];
+  int32_t at = 0;
+  for (int32_t& x : place) {
+    const int32_t count = x;
+    x = at;
+    at += count;
+  }
+  ll.items.resize((size_t)n);
+  for (const Unit& u : units) {
+    const int32_t pos = place[max_unit - (u.page_end - u.page_begin)]++, turn = pos / grid, l = pos - turn * grid;
+    ll.items[(size_t)ll.cta_ptr[turn & 1 ? grid - 1 - l : l] + turn] = make_item(u, u.page_begin, u.page_end);
+  }
+  return true;
+}
+
 // Split-KV decode, short launches: fixed shares with block-local merges.  Whole units are first
 // dealt to thread blocks (largest first, each to the least-loaded block, then units are moved from
 // the fullest block to the emptiest while that lowers the maximum); inside a block its units'
@@ -1480,7 +1518,9 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
     if (f32) {
       // one share per block; whole units while the fullest block stays within the merge launch of the average
       // (a block takes a 16-token page in about 0.1 us, the launch 4 - 5 us)
-      partition(split_units, split_sms * pie_f32_blocks_per_sm(ctx, false), 16, max_rows, true, plan->split, nullptr, ctx->lean ? lean_slack : 45);
+      const int f32_grid = split_sms * pie_f32_blocks_per_sm(ctx, false);
+      if (!deal_in_turns(split_units, f32_grid, max_rows, plan->split))
+        partition(split_units, f32_grid, 16, max_rows, true, plan->split, nullptr, ctx->lean ? lean_slack : 45);
       plan->split.n_static = (int32_t)plan->split.items.size();
     } else if (int c_blocks = 0, c_warps = 0; pick_cluster(ctx, split_units, plain_units, W, split_sms, hp, plan->overlap, long_launch, &c_blocks, &c_warps)) {
       partition_cluster(split_units, c_blocks, c_warps, P == 8 ? 2 : 1, max_rows, plan->split);

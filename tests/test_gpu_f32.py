@@ -74,3 +74,16 @@ def test_fp32_hidden_rows_may_hold_anything(D, P, bad):
         assert (info["num_simple_rows"] == 0) == (flags == 0)
         assert np.abs(O[~sees] - clean[0][~sees]).max() <= TOL and np.abs(L[~sees] - clean[1][~sees]).max() <= TOL
         assert np.isnan(O[sees]).all()
+
+
+def test_fp32_thousands_of_units():
+    """Many short decodes: units dealt to the blocks by size, there and back, with every count left over."""
+    from tests._util import SmallBatch, oracle_on, random_seqs
+    from tests.test_gpu_matrix import run_gpu
+    rng = np.random.RandomState(6)
+    args = SmallBatch(random_seqs(rng, [(1, int(n)) for n in rng.randint(1, 25, 1301)], 8, 4, 64), 8).paged(8, order="random", seed=6)
+    gpu_args = dict(args, pool={p: (k.copy(), v.copy()) for p, (k, v) in args["pool"].items()})
+    O_ref, L_ref = oracle_on(args)
+    O, L, info = run_gpu(gpu_args, max(args["pool"]) + 1, 4, 64, "f32")
+    assert info["num_split_items"] == 1301 * 4 and info["num_merge_groups"] == 0
+    assert np.abs(O - O_ref).max() <= TOL and np.abs(L - L_ref).max() <= TOL
