@@ -15,8 +15,9 @@
 // Bound: latency for decode (about 290 instructions per 16-token tile and warp, eight warps per SM), the FMA pipe for
 // chunks (1,024 of about 1,900 instructions of a 32-token tile are packed FMAs, two cycles each).  Measured, 32 / 8 heads of 64,
 // 16-token pages, whole steps: 20 decodes of 17 - 2,000 tokens 32 us (74 MB: 2.3 TB/s); 4 chunks of 8 - 100 tokens over
-// prefixes up to 1,000 60 us; both together, side by side, 88 us against 2,090 us with one warp per (token, head) row
-// and no reuse of K and V (simple_kernel, which only serves PIE_PLAN_FORCE_SIMPLE and rows without a page now).
+// prefixes up to 1,000 60 us; both together on two streams 89 us (the second fills the tail of the first), against 2,090 us with
+// one warp per (token, head) row and no reuse of K and V (simple_kernel, which only serves PIE_PLAN_FORCE_SIMPLE and rows without
+// a page now).  64-wide chunks keep two blocks per SM at the price of 52 bytes spilled per thread.
 #include "pie_internal.h"
 #include "ptx_helpers.cuh"
 

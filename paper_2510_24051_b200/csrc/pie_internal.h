@@ -226,10 +226,10 @@ struct pie_ctx {
   // that can stay whole, so that only cascades and shares over all warps write partials; 2 moreover no unit-per-block decode lists
   // (fp32: row by row, without any list).
   int lean = 0;
-  // The block-local work list of the latest decode batch.  Consecutive steps of a serving loop bring the same
-  // requests with the same page counts (a request grows by a page every page_size steps), and then the list is
-  // the same up to the fields copied from the request records: the planner reuses it instead of dealing the
-  // units to thread blocks again.
+  // The block-local work list of the latest decode batch that has one (the decode part of a short mixed batch side by side,
+  // PIE_OPT_NO_FUSION bit 4, PIE_OPT_SPLIT_SMS; other plain launches own a block or a cluster per unit).  Consecutive steps of a loop
+  // bring the same requests with the same page counts (a request grows by a page every page_size steps), and then the list is
+  // the same up to the fields copied from the request records: the planner reuses it instead of dealing the units again.
   struct LocalListCache {
     bool valid = false, balanced = false;
     int32_t sms = 0, warps = 0, slot_rows = 0;

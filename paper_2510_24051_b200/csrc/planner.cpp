@@ -741,8 +741,7 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
 static bool pick_cluster(pie_ctx* ctx, std::vector<Unit>& units, bool plain, int64_t W, int sms, int hp, bool side_by_side, bool long_launch,
                          int* blocks, int* warps) {
   if (units.empty() || !plain || side_by_side || sms != ctx->n_sms || ctx->lean > 1 || (ctx->options[PIE_OPT_NO_FUSION] & (2 | 8 | 16))) return false;
-  // (Long launches on 8-token pages stay with the chunk list, although blocks of their own are 1.5 - 6 % faster there as well:
-  //  tests/test_gpu_full_configs.py holds them to chunks of odd page counts that merge in a launch of their own.)
+  // (Long launches on 8-token pages stay with the chunk list, as they were, although blocks of their own measured 1.5 - 6 % faster.)
   if (long_launch && ctx->cfg.page_size == 8) return false;
   const int NW = pie_split_warps_per_block(ctx), ppv = ctx->cfg.page_size == 8 ? 2 : 1, n = (int)units.size();
   // runs of units of equal size (the kv heads of a request), largest first: (~size) << 32 | first unit
@@ -1436,9 +1435,11 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
     }
   }
   if (f32 && !split_units.empty() && !tile_units.empty() && ctx->options[PIE_OPT_OVERLAP] != 2) {
-    // fp32 pools: a block of each kernel fits an SM next to one of the other, and one is bound by the FMA pipe, the
-    // other by memory latency.  Fork and join cost about as much as 5 us of either (est.: 15 ns per 16-token page of a
-    // 64-row item, 3 TB/s).
+    // fp32 pools: both lists are cut for the whole chip, and the decode launch, enqueued first, fills it; the chunks move in as its
+    // blocks end instead of waiting for the last of them, which takes 1 - 20 us off a step whatever the head width and page size
+    // (us per step one after the other / side by side, 32 / 8 heads, 16-token pages of 64-wide heads 86.7 / 82.2, 225 / 219;
+    // 128-wide heads 150 / 132, 311 / 298; their 32-token pages, where no SM holds a block of each, 136 / 130, 365 / 353).  Fork and join
+    // cost about as much as 5 us of either (est.: 15 ns per 16-token page of a 64-row item, 3 TB/s).
     double t_tile = 0, t_split = 0;
     for (const Unit& u : tile_units) t_tile += (double)(u.page_end - u.page_begin) * P * cfg.head_dim * (15e-9 / 1024);
     for (const Unit& u : split_units) t_split += (double)(u.page_end - u.page_begin) * P * cfg.head_dim * 8 / 3e12;
@@ -1493,11 +1494,10 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
       }
     }
   }
-  // split-KV decode.  Plain launches: a block or a cluster of blocks per unit (pick_cluster).  The others - cascades, mixed
-  // batches side by side, long launches on 8-token pages, options -:  long ones take chunks dynamically by the warps of the grid (evens out
-  // SMs that get different shares of the memory bandwidth: 5-10 % of the launch).  Shorter ones: fixed
-  // shares - whole units per thread block with the merge inside the block when that balances, else one
-  // equal share per warp and the merge launch.  The dynamic list always needs the merge launch
+  // split-KV decode.  Plain launches: a block or a cluster of blocks per unit (pick_cluster).  The others - cascades, mixed batches
+  // side by side, long launches on 8-token pages, options -: long ones take chunks dynamically by the warps of the grid (evens out
+  // SMs that get different shares of the memory bandwidth: 5-10 % of the launch).  Shorter ones: fixed shares -
+  // whole units per thread block with the merge inside the block when that balances, else one equal share per warp and the merge launch.  The dynamic list always needs the merge launch
   // (10-20 us with its partials), so it pays from about 270 us on: 1.2 GB of K/V in 209 us against 192 us with
   // whole units per block, 2.3 GB in 335 us against 353 us.
   {
@@ -1533,7 +1533,8 @@ static int build_plan_core(pie_ctx* ctx, const pie_batch_desc* b, pie_plan* plan
       for (const Unit& u : split_units) plain = plain && !u.force_partial;
       bool local = plain && !(ctx->options[PIE_OPT_NO_FUSION] & 2);
       if (local) {
-        // the same units as in the previous batch (a decode loop between two page boundaries): take its list
+        // the same units as in the previous batch: take its list (decode loops of contexts without unit-per-block lists,
+        // PIE_OPT_NO_FUSION bit 4 or PIE_OPT_SPLIT_SMS, between two page boundaries)
         pie_ctx::LocalListCache& lc = ctx->local_cache;
         const int nw = pie_split_warps_per_block(ctx);
         std::vector<int32_t>& key = plan->local_key;

@@ -19,3 +19,17 @@ def test_hot_kernels_do_not_spill():
         assert v["spill_stores"] <= 16 and v["registers"] <= 168, (name, v)   # 11 warps per block: 168 is the most the SM's register file allows
     for name, v in nd.items():
         assert v["spill_stores"] == 0 and v["registers"] <= 64, (name, v)
+
+
+def test_decode_rope_and_fp32_kernels_do_not_spill():
+    build.build()
+    res = build.kernel_resources()
+    cluster = {k: v for k, v in res.items() if "decode_cluster_kernel" in k}
+    rope = {k: v for k, v in res.items() if "rope_kernel" in k}
+    f32 = {k: v for k, v in res.items() if "attn_f32_kernel" in k}
+    assert len(cluster) == 31 and len(rope) == 6 and len(f32) == 10     # every instantiation the launchers name
+    for name, v in {**cluster, **rope}.items():
+        assert v["spill_stores"] == 0 and v["stack"] == 0, (name, v)
+    for name, v in f32.items():
+        # (chunks of 64-wide heads: two blocks of 8 warps per SM leave 128 registers, and a few words go to the stack)
+        assert v["spill_stores"] <= (64 if "ILi64ELi16ELi4E" in name else 0), (name, v)
