@@ -14,7 +14,8 @@ region is reported (with the fastest and slowest one beside it).
 With no `--workload` the run covers every baseline configuration in one go and prints ONE JSON
 line: the top level describes the headline workload (the largest single-GPU configuration,
 `long_context_policy`) and `workloads` holds one entry per configuration - each with its own
-step time, tokens/s, roofline of its dominant kernel, end-to-end figure, clocks and CPU baseline.
+step time, tokens/s, roofline of its dominant kernel, end-to-end figure, clocks and CPU baseline (in
+short: all that was measured for them, with the words that go with it, is one JSON line on stderr).
 
 The `e2e` figure goes through pie_forward_host: planning, pinned-host -> device copies of
 Q/K/V and the device -> host read of the outputs are inside its timed region.  For decode
@@ -263,6 +264,29 @@ def run_reference(args):
         "e2e": {"value": val, "unit": "tokens/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0},
         "gpu_launches": 0,
     }))
+
+
+def rounded(x):
+    """Floats to six digits: a line of all workloads with full ones outgrows what readers of logs keep of a line."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: rounded(v) for k, v in x.items()}
+    return [rounded(v) for v in x] if isinstance(x, list) else x
+
+
+def brief(e):
+    """A workload's entry in the printed line: the figures, without the headline's prose."""
+    keys = {"roofline": ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic", "algorithmic_bytes", "useful_flops"), "cpu_baseline": ("value", "unit", "cores", "kind"),
+            "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step"), "clocks": ("sm_mhz", "sm_max_mhz", "reasons"),
+            "config": ("workload", "requests", "query_tokens", "rows", "vocab", "heads", "head_dim", "page_size")}
+    out = {k: e[k] for k in ("timed", "value", "unit", "ms_per_step", "ms_per_step_min", "ms_per_step_max", "dtype", "hbm_gbs_step", "useful_flops_step", "plan_ms", "gpu_launches") if k in e}
+    for k, names in keys.items():
+        if isinstance(e.get(k), dict):
+            out[k] = {n: e[k][n] for n in names if n in e[k]}
+    if "kernel_ms" in e:
+        out["kernel_ms"] = {k: v for k, v in e["kernel_ms"].items() if v}
+    return out
 
 
 class Env:
@@ -806,10 +830,11 @@ def main():
         if args.workload == "all":
             if env.world == 1:
                 entries["tiny_fp32"] = {"timed": False, "note": "correctness-only configuration (fp32, 4 requests): covered by the parity tests"}
-            line["workloads"] = entries
+            line["workloads"] = {name: brief(e) for name, e in entries.items()}
+            print(json.dumps({"workloads": entries}), file=sys.stderr)      # (everything measured; the line below has to stay short)
         line["device"] = device
         line["wall_seconds"] = time.perf_counter() - t_start
-        print(json.dumps(line))
+        print(json.dumps(rounded(line), separators=(",", ":")))
     env.close()
 
 
